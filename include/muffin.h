@@ -85,8 +85,11 @@ typedef struct {
                          (starlet, B3 spline, periodic) with J = levels <= 4
                          scales, K = J + 1 planes, ||W_s||^2 = 1 */
   int32_t precision;  /* arithmetic of the spectral DCT W_lambda (Sec. 4.2.1):
-                         0 (default) = dense L x L products as 3xTF32 split
-                         products on the tensor cores, FP32 accumulation;
+                         0 (default) = the fastest form with FP32 accuracy:
+                         64 bands as 3xTF32 split products on the tcgen05
+                         tensor cores with FP32 accumulation, other powers
+                         of two as the fast DCT-II of 1, other counts as
+                         dense FP32 products folded about the middle band;
                          1 = FP32 on the CUDA cores by a fast DCT-II
                          (Makhoul's reordering into one complex DFT per
                          pixel, O(L log L)); needs nbands a power of two in
@@ -192,7 +195,7 @@ MUFFIN_API muffin_status muffin_plan_weights_from_x0(muffin_plan plan, const flo
 /* ---- per-shape tuning (launch variants of the hot kernels)
  *
  * For 64-band plans the tuner also times the two spectral kernels (tcgen05
- * and mma.sync), whose results agree to FP32 accuracy.  Two further launch
+ * and dense FP32), whose results agree to FP32 accuracy.  Two further launch
  * choices change speed but not results (every variant computes the same
  * sums in the same order, so outputs are bit-identical):
  *   syn_packed       bit 0: coarse wavelet synthesis levels, bit 1: level 1;
@@ -203,7 +206,7 @@ MUFFIN_API muffin_status muffin_plan_weights_from_x0(muffin_plan plan, const flo
  * Which is fastest depends on the cube shape and the GPU. */
 typedef struct {
   int32_t syn_packed;      /* chosen synthesis variant bits */
-  int32_t dct_ctas_per_sm; /* chosen grid of the mma.sync spectral kernel (0 = all resident) */
+  int32_t dct_ctas_per_sm; /* chosen grid of the dense spectral kernel (0 = a CTA per tile) */
   int32_t spectral_tcgen05;/* 1: spectral step on tcgen05 (64-band plans, see
                               muffin_plan_set_spectral_kernel) */
   int32_t from_cache;      /* 1: taken from the in-process or file cache */
@@ -234,9 +237,8 @@ MUFFIN_API muffin_status muffin_plan_autotune(muffin_plan plan, const char *cach
 
 /* Spectral step kernel for plans with 64 bands: 1 (default for L = 64) runs
  * it on the tcgen05 tensor cores (tensor-memory accumulators, operands in
- * shared memory), 0 on the warp-level mma.sync kernel used for other band
- * counts.  Both compute the same 3xTF32 products; their FP32 rounding order
- * differs, so results agree to FP32 accuracy, not bit for bit.  Drops
+ * shared memory, 3xTF32 products), 0 on the dense FP32 kernel used for band
+ * counts that are no power of two.  Their rounding differs, so results agree to FP32 accuracy, not bit for bit.  Drops
  * captured graphs and the iterate state.  Errors: EINVAL (NULL plan, or 1
  * with L != 64). */
 MUFFIN_API muffin_status muffin_plan_set_spectral_kernel(muffin_plan plan, int32_t tcgen05);
@@ -262,8 +264,8 @@ MUFFIN_API muffin_status muffin_plan_set_tuning(muffin_plan plan, int32_t syn_pa
  * order; both variants stay within the same tolerance of the oracle). */
 typedef struct {
   int32_t syn_packed;       /* synthesis row-pass variant bits, 0..3 */
-  int32_t dct_ctas_per_sm;  /* mma.sync spectral grid, 0 = all resident */
-  int32_t spectral_tcgen05; /* 64-band plans: 1 tcgen05, 0 mma.sync */
+  int32_t dct_ctas_per_sm;  /* dense spectral kernel: persistent grid, 0 = a CTA per tile */
+  int32_t spectral_tcgen05; /* 64-band plans: 1 tcgen05, 0 the dense FP32 kernel */
   int32_t grad_chunk;       /* images per pass of the gradient's three FFT
                                passes: 0 = each pass over all images of a
                                chain group; k > 0 = the three passes run k
@@ -556,7 +558,7 @@ MUFFIN_API muffin_status muffin_op_analysis(muffin_plan plan, const float *x, fl
 /* x = W_s^T u (synthesis summed over the K bases). */
 MUFFIN_API muffin_status muffin_op_synthesis(muffin_plan plan, const float *u, float *x);
 /* v^n = C x^n for every pixel (inverse = 0) or x^n = C^T v^n (inverse = 1),
- * C the orthonormal DCT-II (3xTF32 tensor-core products). */
+ * C the orthonormal DCT-II. */
 MUFFIN_API muffin_status muffin_op_dct(muffin_plan plan, const float *x, float *v,
                             int32_t inverse);
 

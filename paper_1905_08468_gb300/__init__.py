@@ -158,7 +158,7 @@ class Plan:
 
     def set_spectral_kernel(self, tcgen05: bool) -> None:
         """Spectral step on the tcgen05 tensor cores (64-band plans) or on
-        the mma.sync kernel."""
+        the dense FP32 kernel."""
         native.check(self._lib.muffin_plan_set_spectral_kernel(self._h, int(bool(tcgen05))))
 
     def inject_timeout(self, on: bool) -> None:

@@ -1,4 +1,5 @@
-// Spectral step in FP32 on the CUDA cores (plans created with precision 1).
+// Spectral step in FP32 on the CUDA cores: plans created with precision 1, and
+// every power-of-two band count but 64.
 //
 // The same updates as the tensor-core kernels (Alg. 2 eqs. vt, v, upt and the
 // derivative forms of Algs. 3/4), with the orthonormal DCT-II of each pixel
@@ -15,7 +16,13 @@
 // spectra, and before the inverse their Hermitian spectra are merged, so
 // one DFT of length L serves two pixel spectra each way.  The DFTs are the
 // shared-memory Stockham transforms of the gradient passes.  The work is
-// O(L log L) per pixel, so the step is bound by its HBM traffic at every L.
+// O(L log L) per pixel, so the step is bound by its HBM traffic at every L
+// (512 x 512 x 256, one chain: 0.28 ms, 4.8 TB/s; the dense 3xTF32 product on
+// mma.sync took 1.74 ms).  Images with few tiles run 64-thread CTAs with a
+// quarter of the pixels (64 x 64 x 32, three chains: 24.8 -> 17.6 us).  The old
+// duals of a chain are requested before the chain's forward DFT (512 x 512 x
+// 32, three chains: 165 -> 134 us), and chain 2's gamma v'_gamma + v is formed
+// after the inverse DFTs, which are linear, so no dual stays in a register.
 //
 // A CTA owns a tile of PT = 2 NB pixels of one cube.  Phases: load z = 2 x~ -
 // x of every band of the tile (float2 pairs of pixels, coalesced along the
@@ -35,9 +42,9 @@ namespace muffin {
 
 namespace {
 
-constexpr int FT = 256;   // threads per CTA
-
-template <int L>
+// FT threads per CTA: 256, or 64 where the tiles of 256-thread CTAs are too
+// few for the SMs
+template <int L, int FT>
 struct FShape {
   static constexpr int VPT = fft_vpt(L);
   static constexpr int NB0 = FT * VPT / L;            // sequences the DFT threads cover
@@ -47,7 +54,9 @@ struct FShape {
   static constexpr int PITCH = ((L - 1) + (L - 1) / 16 + 1) | 1;
   static constexpr int NTASK = NB * (L / 2);
   static constexpr int TPT = (NTASK + FT - 1) / FT;   // tasks per thread
+  static constexpr int KS = FT / NB;                  // band pairs between a thread's tasks
   static_assert(NB * L / VPT <= FT, "the DFT threads fit in the CTA");
+  static_assert(FT % NB == 0, "a thread keeps one pixel pair");
   static_assert(TPT * 4 <= 32, "mask bits of a thread's tasks fit in 32 bits");
 };
 
@@ -78,9 +87,9 @@ __device__ __forceinline__ int mpos(int l) {
   return (l & 1) ? L - 1 - (l >> 1) : (l >> 1);
 }
 
-template <int L, int CH, int MODE>
-__global__ void __launch_bounds__(FT, 2) k_dct_f32(F32Args a) {
-  using S = FShape<L>;
+template <int L, int CH, int MODE, int FT>
+__global__ void __launch_bounds__(FT, FT == 64 ? 6 : 2) k_dct_f32(F32Args a) {
+  using S = FShape<L, FT>;
   constexpr int NB = S::NB, PT = S::PT, PITCH = S::PITCH;
   extern __shared__ float2 fsm[];
   float2 *tw = fsm;                 // DFT stage twiddles
@@ -133,51 +142,41 @@ __global__ void __launch_bounds__(FT, 2) k_dct_f32(F32Args a) {
       for (int c = 0; c < CH; ++c) dat[c * NB * PITCH + o] = z[c];
     }
   }
-  // one chain: the old duals and the pixel weights of this thread's tasks,
-  // requested now so that their latency is covered by the forward DFT
-  // (three chains have no registers to spare for it)
-  constexpr bool PREF = MODE == WAVE_ITERATE && CH == 1;
-  constexpr int PF = PREF ? S::TPT : 1;
-  float2 pv1[PF], pv2[PF], pal[PF];
-  if constexpr (PREF) {
+  // a thread's tasks share its pixel pair; the old duals of a chain are
+  // requested before the chain's forward DFT, which covers their latency
+  const int ps = tid % NB, kk0 = tid / NB;
+  const size_t pix = n0 + 2 * ps;
+  const bool valid = pix < N;
+  constexpr int TPT = MODE == WAVE_ITERATE ? S::TPT : 1;
+  float2 pv1[TPT], pv2[TPT], al = make_float2(0.f, 0.f);
+  // (a pixel block of the sharded form starts anywhere: no vector load)
+  if (MODE == WAVE_ITERATE && valid) al = make_float2(alpha[pix], alpha[pix + 1]);
+  auto duals = [&](int c) {
 #pragma unroll
-    for (int r = 0; r < S::TPT; ++r) {
-      const int it = tid + r * FT;
-      pv1[r] = pv2[r] = pal[r] = make_float2(0.f, 0.f);
-      if (it < S::NTASK) {
-        const int s = it % NB, kk = it / NB;
-        const int k1 = kk, k2 = kk ? L - kk : L / 2;
-        const size_t pix = n0 + 2 * s;
-        if (pix < N) {
-          pv1[r] = ld2(a.v + cb + (size_t)k1 * N + pix);
-          pv2[r] = ld2(a.v + cb + (size_t)k2 * N + pix);
-          pal[r] = ld2(alpha + pix);
-        }
+    for (int r = 0; r < TPT; ++r) {
+      const int kk = kk0 + r * S::KS;
+      pv1[r] = pv2[r] = make_float2(0.f, 0.f);
+      if (tid + r * FT < S::NTASK && valid) {
+        const float *vp = a.v + c * CS + cb + pix;
+        pv1[r] = ld2(vp + (size_t)kk * N);
+        pv2[r] = ld2(vp + (size_t)(kk ? L - kk : L / 2) * N);
       }
     }
-  }
-  if (!inv_op) {
-    __syncthreads();
-#pragma unroll 1
-    for (int c = 0; c < CH; ++c) fft_inplace<L, false>(dat + c * NB * PITCH, NB, PITCH, tw);
-  } else {
-    __syncthreads();   // tables
-  }
+  };
 
   // ---- per (pixel pair, band pair) tasks
   uint32_t mask = 0;
-  float keep0[CH == 3 ? S::TPT : 1][4];
 #pragma unroll 1
   for (int c = 0; c < CH; ++c) {
     float2 *d = dat + c * NB * PITCH;
+    if (MODE == WAVE_ITERATE) duals(c);
+    if (c == 0) __syncthreads();   // tables and the tile
+    if (!inv_op) fft_inplace<L, false>(d, NB, PITCH, tw);
 #pragma unroll
     for (int r = 0; r < S::TPT; ++r) {
-      const int it = tid + r * FT;
-      if (it >= S::NTASK) break;
-      const int s = it % NB, kk = it / NB;
+      if (tid + r * FT >= S::NTASK) break;
+      const int s = ps, kk = kk0 + r * S::KS;
       const int k1 = kk, k2 = kk ? L - kk : L / 2;
-      const size_t pix = n0 + 2 * s;
-      const bool valid = pix < N;
       const float2 w = mk[kk];
       // orthonormal coefficients X[k1], X[k2] of pixels A (.x) and B (.y)
       float2 X1 = make_float2(0.f, 0.f), X2 = X1;
@@ -206,20 +205,10 @@ __global__ void __launch_bounds__(FT, 2) k_dct_f32(F32Args a) {
         Y1 = valid ? ld2(a.in + cb + (size_t)k1 * N + pix) : make_float2(0.f, 0.f);
         Y2 = valid ? ld2(a.in + cb + (size_t)k2 * N + pix) : make_float2(0.f, 0.f);
       } else {
-        float2 al;
-        if constexpr (PREF) al = pal[r];
-        else al = valid ? ld2(alpha + pix) : make_float2(0.f, 0.f);
         const float sa = (c == 2) ? sigma : sigma * gamma;
         float *v1p = a.v + c * CS + cb + (size_t)k1 * N + pix;
         float *v2p = a.v + c * CS + cb + (size_t)k2 * N + pix;
-        float2 o1, o2;
-        if constexpr (PREF) {
-          o1 = pv1[r];
-          o2 = pv2[r];
-        } else {
-          o1 = valid ? ld2(v1p) : make_float2(0.f, 0.f);
-          o2 = valid ? ld2(v2p) : make_float2(0.f, 0.f);
-        }
+        const float2 o1 = pv1[r], o2 = pv2[r];
         float vt[4] = {fmaf(sa * al.x, X1.x, o1.x), fmaf(sa * al.y, X1.y, o1.y),
                        fmaf(sa * al.x, X2.x, o2.x), fmaf(sa * al.y, X2.y, o2.y)};
         float vn[4];
@@ -236,15 +225,6 @@ __global__ void __launch_bounds__(FT, 2) k_dct_f32(F32Args a) {
         if (valid) {
           st2(v1p, make_float2(vn[0], vn[1]));
           st2(v2p, make_float2(vn[2], vn[3]));
-        }
-        if constexpr (CH == 3) {
-          if (c == 0) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) keep0[r][e] = vn[e];
-          } else if (c == 2) {   // gamma v'_gamma + v
-#pragma unroll
-            for (int e = 0; e < 4; ++e) vn[e] = fmaf(gamma, vn[e], keep0[r][e]);
-          }
         }
         Y1 = make_float2(vn[0], vn[1]);
         Y2 = make_float2(vn[2], vn[3]);
@@ -274,18 +254,19 @@ __global__ void __launch_bounds__(FT, 2) k_dct_f32(F32Args a) {
   // ---- back in band order: t (iteration) or C^T in (operator)
 #pragma unroll 4
   for (int it = tid; it < L * NB; it += FT) {
-    const int s = it % NB, l = it / NB;
-    const size_t pix = n0 + 2 * s;
-    if (pix >= N) continue;
-    const int o = s * PITCH + fpad(mpos<L>(l));
+    const int l = it / NB;
+    if (!valid) continue;
+    const int o = ps * PITCH + fpad(mpos<L>(l));
     const size_t j = cb + (size_t)l * N + pix;
     if (MODE == WAVE_TRANSFORM) {
       st2(a.out + j, dat[o]);
     } else {
-      const float2 al = ld2(alpha + pix);
+      const float2 w0 = dat[o];
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
-        const float2 val = dat[c * NB * PITCH + o];
+        float2 val = c == 0 ? w0 : dat[c * NB * PITCH + o];
+        if (c == 2)    // C^T (gamma v'_gamma + v)
+          val = make_float2(fmaf(gamma, val.x, w0.x), fmaf(gamma, val.y, w0.y));
         const float s2 = (c == 2) ? 1.f : gamma;
         st2(a.t + c * CS + j, make_float2(s2 * al.x * val.x, s2 * al.y * val.y));
       }
@@ -293,13 +274,13 @@ __global__ void __launch_bounds__(FT, 2) k_dct_f32(F32Args a) {
   }
 }
 
-template <int L, int CH, int MODE>
-cudaError_t launch_f32(const F32Args &a, cudaStream_t st, Prof *prof) {
-  using S = FShape<L>;
+template <int L, int CH, int MODE, int FT>
+cudaError_t launch_f32_t(const F32Args &a, cudaStream_t st, Prof *prof) {
+  using S = FShape<L, FT>;
   const size_t sm = (size_t)(a.tw_len + L + CH * S::NB * S::PITCH) * sizeof(float2);
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_dct_f32<L, CH, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_dct_f32<L, CH, MODE, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          200 * 1024);
     attr = true;
   }
@@ -309,8 +290,15 @@ cudaError_t launch_f32(const F32Args &a, cudaStream_t st, Prof *prof) {
                (MODE == WAVE_ITERATE ? 2.0 : 1.0) * CH * vox * (2.5 * std::log2((double)L) + 6.0),
                st);
   const unsigned gx = (unsigned)((a.npix + S::PT - 1) / S::PT);
-  k_dct_f32<L, CH, MODE><<<dim3(gx, a.B), FT, sm, st>>>(a);
+  k_dct_f32<L, CH, MODE, FT><<<dim3(gx, a.B), FT, sm, st>>>(a);
   return cudaGetLastError();
+}
+
+template <int L, int CH, int MODE>
+cudaError_t launch_f32(const F32Args &a, cudaStream_t st, Prof *prof) {
+  const size_t tiles = (a.npix + FShape<L, 256>::PT - 1) / FShape<L, 256>::PT * a.B;
+  return tiles < 304 ? launch_f32_t<L, CH, MODE, 64>(a, st, prof)
+                     : launch_f32_t<L, CH, MODE, 256>(a, st, prof);
 }
 
 template <int CH, int MODE>

@@ -258,10 +258,11 @@ struct DctArgs {
   int B;                   // cubes in the batch (band-major, cube after cube)
   const float *chi, *clo;  // [Lp][Lp] C split in TF32 hi + lo (zero padded)
   const float *cthi, *ctlo;// [Lp][Lp] C^T split
+  const float *fold;       // tables of the folded dense products (dct_fold_tables)
   const float *alpha;      // [B][n*n] pixel weights
   const DevScalars *sc;    // [B]
-  int ctas_per_sm;         // persistent spectral grid: CTAs per SM (0: max resident)
-  int tc;                  // 1: tcgen05 kernel (L = 64), 0: mma.sync kernel
+  int ctas_per_sm;         // dense kernel: persistent grid of so many CTAs per SM (0: a CTA per tile)
+  int tc;                  // 1: tcgen05 kernel (L = 64), 0: dense kernel
   int *err;                // device flag raised when a tensor-core wait gives up
   int inject_timeout;      // test hook: the tcgen05 kernel issues no products
   int f32;                 // 1: FP32 fast DCT on the CUDA cores (dct_f32.cu)
@@ -282,6 +283,8 @@ cudaError_t dct_op(const DctArgs &d, const float *in, float *out, int inverse,
 cudaError_t dct_dual_f32(const DctArgs &d, const Group &gr, cudaStream_t st);
 cudaError_t dct_op_f32(const DctArgs &d, const float *in, float *out, int inverse,
                        cudaStream_t st);
+int dct_fold_table_len(int L);                       // floats; C: the [L][L] DCT-II matrix
+void dct_fold_tables(int L, const double *C, float *tab);
 int dct_f32_table_len(int L);
 void dct_f32_tables(int L, float2 *tab);
 

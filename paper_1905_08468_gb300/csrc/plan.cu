@@ -136,6 +136,17 @@ muffin_status validate(const muffin_params *p) {
   return MUFFIN_OK;
 }
 
+// Whether the spectral step runs as the FP32 fast DCT: where the caller asks
+// for it, and for every power-of-two band count but 64.  The fast DCT does
+// O(log L) work per voxel and is bound by its memory traffic, while a dense
+// product grows with L (1024 x 1024 x 256, one chain: 1.1 ms against 7.0 ms in
+// 3xTF32) and keeps more error.  At 64 bands the tcgen05 kernel is the faster one
+// with three chains at 1024 x 1024 (0.94 against 1.00 ms) and stays.
+bool spectral_f32(const muffin_params *p) {
+  const int L = p->nbands;
+  return p->precision == 1 || (L >= 2 && L <= 1024 && L != 64 && (L & (L - 1)) == 0);
+}
+
 // copy a caller array (host or device) into dst (device), count floats
 muffin_status fetch(muffin_plan P, const float *src, float *dst, size_t count) {
   const cudaMemcpyKind k = is_device_ptr(src) ? cudaMemcpyDeviceToDevice
@@ -355,7 +366,8 @@ muffin_status plan_alloc_init(muffin_plan P, const float *alpha, const float *be
   CK(P->alloc(&P->clo, LL2));
   CK(P->alloc(&P->cthi, LL2));
   CK(P->alloc(&P->ctlo, LL2));
-  if (P->p.precision == 1) {
+  CK(P->alloc(&P->fold, (size_t)dct_fold_table_len(L)));
+  if (P->spec_f32) {
     P->ftw_len = dct_f32_table_len(L) - L;
     CK(P->alloc(&P->ftab, (size_t)dct_f32_table_len(L)));
   }
@@ -438,8 +450,11 @@ muffin_status plan_alloc_init(muffin_plan P, const float *alpha, const float *be
   CK(cudaMemcpyAsync(P->clo, lo.data(), LL2 * 4, cudaMemcpyHostToDevice, P->ws));
   CK(cudaMemcpyAsync(P->cthi, thi.data(), LL2 * 4, cudaMemcpyHostToDevice, P->ws));
   CK(cudaMemcpyAsync(P->ctlo, tlo.data(), LL2 * 4, cudaMemcpyHostToDevice, P->ws));
-  std::vector<float2> ft(P->p.precision == 1 ? (size_t)dct_f32_table_len(L) : 0);
-  if (P->p.precision == 1) {
+  std::vector<float> fold((size_t)dct_fold_table_len(L));
+  dct_fold_tables(L, C.data(), fold.data());
+  CK(cudaMemcpyAsync(P->fold, fold.data(), fold.size() * 4, cudaMemcpyHostToDevice, P->ws));
+  std::vector<float2> ft(P->spec_f32 ? (size_t)dct_f32_table_len(L) : 0);
+  if (P->spec_f32) {
     dct_f32_tables(L, ft.data());
     CK(cudaMemcpyAsync(P->ftab, ft.data(), ft.size() * sizeof(float2), cudaMemcpyHostToDevice,
                        P->ws));
@@ -797,14 +812,14 @@ size_t estimate_bytes(const muffin_params *p) {
   else
     for (int j = 1; j < p->levels; ++j) ll += C * Lt * K * (n >> j) * (n >> j);
   size_t b = 3 * NL * 16 + Lt * nh * n * 4 + (size_t)(fft32_table_len((int)n, 16) + fft32_table_len((int)n, 8)) * 8 + n * 16 +
-             4 * Lp * Lp * 4 + B * N * 4 + Lt * 4 + B * sizeof(DevScalars) + B * 32 + 4 + 4 +
+             4 * Lp * Lp * 4 + (size_t)dct_fold_table_len((int)L) * 4 + B * N * 4 + Lt * 4 + B * sizeof(DevScalars) + B * 32 + 4 + 4 +
              (kRedSure + 65 * Lt + 6 * (Lt > 4096 ? Lt : 4096)) * 8 + Lt * 8 +
              C * Lt * nh * n * 8 + (ll ? ll : 1) * 4 + 3 * NL * 4 +
              C * NL * (5 + K) * 4;
   if (p->sure) b += 3 * NL * (5 + K) * 4 + 2 * NL * 4 + C * Lt * nh * n * 8 + (ll ? ll : 1) * 4;
   b += monitor_scratch_doubles((int)Lt) * 8;
-  if (p->precision == 1) b += (size_t)dct_f32_table_len((int)L) * 8 + 16;
-  return b + (p->sure ? 40 : 30) * 16;   // 16 bytes of slack per allocation
+  if (spectral_f32(p)) b += (size_t)dct_f32_table_len((int)L) * 8 + 16;
+  return b + (p->sure ? 41 : 31) * 16;   // 16 bytes of slack per allocation
 }
 
 muffin_status create(const muffin_params *p, const float *psf, const float *alpha,
@@ -824,6 +839,7 @@ muffin_status create(const muffin_params *p, const float *psf, const float *alph
   P->n = p->n; P->L = p->nbands; P->J = p->levels;
   P->dict = p->dictionary;
   P->dct_tc = p->nbands == 64 && p->precision == 0 ? 1 : 0;
+  P->spec_f32 = spectral_f32(p);
   P->K = P->dict == 1 ? p->levels + 1 : p->n_wavelets;
   P->wsn2 = P->dict == 1 ? iuwt_norm2(p->n, p->levels) : (double)p->n_wavelets;
   P->B = p->batch; P->Lt = P->B * P->L;

@@ -54,7 +54,9 @@ struct muffin_plan_s {
   float2 *tw32 = nullptr;
   double2 *tw64 = nullptr;
   float *chi = nullptr, *clo = nullptr, *cthi = nullptr, *ctlo = nullptr;
-  float2 *ftab = nullptr;   // FP32 spectral step tables (precision 1)
+  float *fold = nullptr;    // tables of the dense spectral kernel
+  bool spec_f32 = false;    // the spectral step is the FP32 fast DCT
+  float2 *ftab = nullptr;   // its tables
   int ftw_len = 0;
   float *alpha = nullptr, *beta = nullptr;
   muffin::DevScalars *sc = nullptr;   // [B]
@@ -146,10 +148,11 @@ struct muffin_plan_s {
     muffin::DctArgs d{};
     d.n = n; d.L = L; d.Lp = Lp; d.C = C; d.B = B;
     d.chi = chi; d.clo = clo; d.cthi = cthi; d.ctlo = ctlo;
+    d.fold = fold;
     d.alpha = alpha; d.sc = sc;
     d.ctas_per_sm = dct_ctas;
     d.tc = dct_tc; d.err = kerr; d.inject_timeout = inject_timeout;
-    d.f32 = p.precision == 1; d.ftab = ftab; d.ftw_len = ftw_len;
+    d.f32 = spec_f32; d.ftab = ftab; d.ftw_len = ftw_len;
     d.prof = pp();
     return d;
   }

@@ -136,7 +136,7 @@ muffin_status tune(muffin_plan P, Choice *best, muffin_tune_info *info) {
   const double vox = (double)P->NL * P->Cmax * (P->p.sure ? 2 : 1);
   const int reps = vox >= 2e7 ? 3 : (vox >= 1e6 ? 5 : 10);
   Choice cur{};
-  const bool tf32 = P->p.precision == 0;   // the FP32 spectral step has no variants
+  const bool tf32 = P->p.precision == 0;   // a plan that asks for FP32 has no spectral choices
   cur.dct_tc = P->L == 64 && tf32 ? 1 : 0; // the default kernel for 64 bands
   double t_def = 0.0, t_best = 0.0;
   int cand = 0;
