@@ -216,8 +216,8 @@ typedef struct {
   int32_t grad_chunk;      /* chosen gradient chunking (muffin_schedule) */
   int32_t fft_radix;       /* chosen FFT plan */
   int32_t group_order;     /* chosen kernel order of the ADA-PT groups */
-  int32_t ana_ring;        /* chosen analysis U staging */
-  int32_t ana_pipe;        /* chosen level-1 analysis kernel */
+  int32_t ana_ring;        /* always 0 (muffin_schedule) */
+  int32_t ana_pipe;        /* chosen analysis tile height */
 } muffin_tune_info;
 
 /* Times each candidate configuration on this plan's own buffers (a few
@@ -238,8 +238,8 @@ MUFFIN_API muffin_status muffin_plan_autotune(muffin_plan plan, const char *cach
 /* Spectral step kernel for plans with 64 bands: 1 (default for L = 64) runs
  * it on the tcgen05 tensor cores (tensor-memory accumulators, operands in
  * shared memory, 3xTF32 products), 0 on the dense FP32 kernel used for band
- * counts that are no power of two.  Their rounding differs, so results agree to FP32 accuracy, not bit for bit.  Drops
- * captured graphs and the iterate state.  Errors: EINVAL (NULL plan, or 1
+ * counts that are no power of two.  Their rounding differs, so results
+ * agree to FP32 accuracy, not bit for bit.  Drops captured graphs and the iterate state.  Errors: EINVAL (NULL plan, or 1
  * with L != 64). */
 MUFFIN_API muffin_status muffin_plan_set_spectral_kernel(muffin_plan plan, int32_t tcgen05);
 
@@ -278,19 +278,11 @@ typedef struct {
                                phase, 2 = the two groups concurrently on two
                                streams, each with its own scratch (identical
                                results) */
-  int32_t ana_ring;         /* analysis of the levels specialised for 512,
-                               1024 and 2048 px: 0 = the dual update's U
-                               values loaded by each thread, 1 = the U detail
-                               tiles staged two steps ahead in a shared-memory
-                               ring by cp.async (3 CTAs per SM instead of 4;
-                               identical results) */
-  int32_t ana_pipe;         /* level-1 analysis of an iteration (levels > 1):
-                               0 (default) = basis-major steps with two
-                               barriers each; 1 = chain-major steps with the
-                               row pass of one step and the column pass +
-                               dual update of the previous one in the same
-                               phase (two lo/hi buffers, one barrier per
-                               step); identical results */
+  int32_t ana_ring;         /* 0 or 1, kept for stored schedules: the analysis
+                               has one way to stage U, so it has no effect */
+  int32_t ana_pipe;         /* tile height of the analysis levels (16 or 8
+                               rows): 0 (default) = by the number of tiles,
+                               1 = the other one; identical results */
 } muffin_schedule;
 
 /* Reads / sets the schedule (set drops captured graphs and the iterate

@@ -220,11 +220,10 @@ struct WaveArgs {
   float *scratch;          // LL scratch: level j (1 <= j < J) holds
                            // [C][L][K][n>>j][n>>j] at scratch + lvl_off[j]
   size_t lvl_off[16];
+  uint32_t *masks;         // three chains: masks of the level-1 duals, n^2 K / 8 bytes a
+                           // band (the gradient's spectrum scratch, free by then)
   int dict;                // 0: union of K Daubechies bases, 1: IUWT (K = J + 1 planes)
-  int ana_ring;            // analysis of the size-specialised levels: 1 stages the
-                           // U detail tiles in a shared-memory ring by cp.async
-  int ana_pipe;            // level-1 analysis (iteration, J > 1): 1 runs the
-                           // chain-major kernel with one barrier per step
+  int ana_pipe;            // analysis: 1 takes the other tile height than the rule's
   int syn_packed;          // synthesis variant: bit 0 coarse levels, bit 1
                            // level 1 (0 scalar row pass, 1 packed row pairs)
   Prof *prof;              // optional per-kernel timing

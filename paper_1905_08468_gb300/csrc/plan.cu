@@ -213,6 +213,7 @@ muffin_status iterate_kernels(muffin_plan P, const Group &g, int c0, int c1,
                      P->pp(), P->grad_chunk, P->fft_radix));
   w.L = Lv;
   w.scratch = ll;
+  w.masks = reinterpret_cast<uint32_t *>(S);
   CK(wavelet_synthesis_prox(w, h, P->p.positivity, st));
   CK(wavelet_analysis_dual(w, h, st));
   d.B = c1 - c0;

@@ -87,8 +87,8 @@ struct muffin_plan_s {
   bool profiling = false;
   bool use_graphs = true;
   int syn_packed = 0;     // synthesis variant bits (see WaveArgs::syn_packed)
-  int ana_ring = 0;       // analysis U staging (see WaveArgs::ana_ring)
-  int ana_pipe = 0;       // level-1 analysis kernel (see WaveArgs::ana_pipe)
+  int ana_ring = 0;       // kept for stored schedules, no effect
+  int ana_pipe = 0;       // analysis tile height (see WaveArgs::ana_pipe)
   int dct_ctas = 0;       // spectral kernel CTAs per SM (0: all resident)
   int dct_tc = 0;         // spectral step on tcgen05 (L = 64)
   int grad_chunk = 0;     // images per pass of the gradient FFTs (0: all at once)
@@ -137,9 +137,9 @@ struct muffin_plan_s {
     muffin::WaveArgs w{};
     w.n = n; w.L = Lt; w.Lc = L; w.K = K; w.J = J; w.C = C; w.dict = dict;
     w.beta = beta; w.sc = sc; w.scratch = llscr;
+    w.masks = reinterpret_cast<uint32_t *>(S);
     for (int j = 0; j < 16; ++j) w.lvl_off[j] = lvl_off[j];
     w.syn_packed = syn_packed;
-    w.ana_ring = ana_ring;
     w.ana_pipe = ana_pipe;
     w.prof = pp();
     return w;

@@ -26,8 +26,8 @@ struct Choice {
   int grad_chunk = 0;  // images per pass of the gradient FFTs (0: all)
   int fft_radix = 16;  // largest radix of the gradient FFT plan
   int group_order = 0; // ADA-PT groups: 0 one after the other, 1 phase by phase, 2 two streams
-  int ana_ring = 0;    // analysis U staging in a shared-memory ring
-  int ana_pipe = 0;    // level-1 analysis: chain-major, one barrier per step
+  int ana_ring = 0;    // kept for stored schedules, no effect
+  int ana_pipe = 0;    // analysis tiles of the other height than the rule's
 };
 
 std::mutex g_mu;
@@ -189,18 +189,7 @@ muffin_status tune(muffin_plan P, Choice *best, muffin_tune_info *info) {
     ++cand;
     if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
   }
-  // the analysis U ring, where the size-specialised analysis runs
-  if ((P->n == 512 || P->n == 1024 || P->n == 2048) && P->J > 1 && P->dict == 0 &&
-      s == MUFFIN_OK) {
-    Choice c = *best;
-    c.ana_ring = 1;
-    double t = 0.0;
-    s = time_choice(P, c, reps, e0, e1, &t);
-    ++cand;
-    if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
-  }
-  // the other level-1 analysis kernel (iterations with more than one level),
-  // after the ring, so that it is timed with the ring choice in place
+  // the other tile height of the analysis levels
   if (P->J > 1 && P->dict == 0 && s == MUFFIN_OK) {
     Choice c = *best;
     c.ana_pipe = 1 - c.ana_pipe;

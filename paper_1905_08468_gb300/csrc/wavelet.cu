@@ -9,12 +9,12 @@
 //                                                            (eqs. stpp, stpu)
 //
 // One level per launch.  A CTA owns a tile of TY x TX coefficients of every
-// subband (2TY x 2TX pixels of the level's input) of one band; level 1 keeps
-// its input tile in shared memory and runs all K bases on it, so x~ and x are
-// read once for the 8 bases; the analysis of coarser levels runs one basis
-// per CTA on the approximation left in an LL scratch by the previous level,
-// and every synthesis CTA walks all K bases of its tile (so its copy
-// pipeline stays full across the bases).  Periodic
+// subband (2TY x 2TX pixels of the level's input) of one band; every synthesis
+// CTA walks all K bases of its tile (so its copy pipeline stays full across the
+// bases); coarser levels leave and read approximations in an LL scratch.  The
+// analysis of all but the smallest levels runs in ana_cols.cu, with the columns
+// of its tile in registers; k_ana here serves the small levels (tile in shared
+// memory, level 1 all bases a CTA, coarser levels one basis a CTA).  Periodic
 // extension is a wrap of the tile's load indices, which also covers levels
 // smaller than a filter (the transform stays the exact periodised one).
 //
@@ -38,6 +38,7 @@
 #include <cuda_runtime.h>
 
 #include "kernels.h"
+#include "wavelet.h"
 
 namespace muffin {
 
@@ -71,15 +72,6 @@ constexpr int QXS = 4;                               // scalar synthesis row ite
 constexpr size_t ana_smem(int ch) {
   return ((size_t)ch * A_RP * A_IP + 2 * A_RP * A_LP) * sizeof(float2);
 }
-// the U-ring variant of the size-specialised analysis: the three detail
-// tiles of the next steps' (basis, chain) arrive by cp.async into a ring of
-// shared-memory slots, RING_AHEAD steps ahead of their dual update
-constexpr int RING_SLOTS = 3, RING_AHEAD = 2;
-constexpr size_t ring_off(int ch) { return (ana_smem(ch) + 15) / 16 * 16; }
-constexpr size_t ring_slot_floats() { return (size_t)3 * TY * TX; }
-constexpr size_t ana_smem_ring(int ch) {
-  return ring_off(ch) + (size_t)RING_SLOTS * ring_slot_floats() * sizeof(float);
-}
 constexpr size_t syn_smem(int) {
   return (size_t)(8 * S_CH * S_CP) * sizeof(float) + (size_t)(2 * TY * S_LP) * sizeof(float2);
 }
@@ -87,17 +79,6 @@ constexpr size_t syn_smem(int) {
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   return __ffma2_rn(a, b, c);
 }
-
-struct AnaArgs {
-  int n, M, L, K, last;
-  int Lc;                       // bands per cube (per-cube scalars sc[l / Lc])
-  const float *in;              // level >= 2: LL_{j-1}; level-1 operator: x
-  const float *xt, *x;          // level-1 iteration inputs
-  float *ll_out;                // LL_j scratch when !last
-  float *u;
-  const float *beta;
-  const DevScalars *sc;
-};
 
 struct SynArgs {
   int n, M, L, K, top, positivity;   // M: output side of this level
@@ -245,10 +226,10 @@ __device__ __forceinline__ void ana_cols_dispatch(int p, const float2 *lo_s,
 
 // U values the thread's column item updates in step (bb, c): subbands DX
 // (low y, high x), DY, HH and, at the last level, LL
-template <int MODE, int NS, int MS>
+template <int MODE>
 __device__ __forceinline__ void ana_prefetch(const AnaArgs &a, int l, int bb, int c,
                                              int kx0, int ky0, float (&pre)[4][QY]) {
-  const int n = NS ? NS : a.n, M = MS ? MS : a.M;
+  const int n = a.n, M = a.M;
   const int h = M >> 1, hn = h * n;
   const int kx = threadIdx.x % TX, s = threadIdx.x / TX;
   const int kxg = kx0 + kx;
@@ -261,23 +242,23 @@ __device__ __forceinline__ void ana_prefetch(const AnaArgs &a, int l, int bb, in
     pre[0][qq] = act ? up[o + h] : 0.f;
     pre[1][qq] = act ? up[o + hn] : 0.f;
     pre[2][qq] = act ? up[o + hn + h] : 0.f;
-    pre[3][qq] = (act && !NS && a.last) ? up[o] : 0.f;
+    pre[3][qq] = (act && a.last) ? up[o] : 0.f;
   }
 }
 
 // dual update p = u + q w, u = sat(p) (or the mask of channel 0) and the
 // stores of step (bb, c)
-template <int MODE, int NS, int MS>
+template <int MODE>
 __device__ __forceinline__ void ana_emit_step(const AnaArgs &a, int l, int bb, int c,
                                               int kx0, int ky0, float q,
                                               const float (&cf)[4][QY],
                                               const float (&pre)[4][QY], uint32_t &keep) {
-  const int n = NS ? NS : a.n, M = MS ? MS : a.M;
+  const int n = a.n, M = a.M;
   const int h = M >> 1, hn = h * n;
   const int kx = threadIdx.x % TX, s = threadIdx.x / TX;
   const int kxg = kx0 + kx;
   float *up = a.u + ((size_t)(c * a.L + l) * a.K + bb) * ((size_t)n * n);
-  const bool last = !NS && a.last;   // specialised sizes never run the last level
+  const bool last = a.last;
   float *llp = last ? nullptr : a.ll_out + ((size_t)(c * a.L + l) * a.K + bb) * h * h;
   const int sbo[4] = {h, hn, hn + h, 0};
   if (c == 0) keep = 0;
@@ -309,18 +290,13 @@ __device__ __forceinline__ void ana_emit_step(const AnaArgs &a, int l, int bb, i
   }
 }
 
-// NS, MS > 0: the image side n and the level's input side M fixed at
-// compile time (levels 1 and 2 of the common sizes), so every U offset of
-// the dual update is an immediate
-template <int CH, int MODE, bool LEVEL1, int NS, int MS, bool RING = false>
-__global__ void __launch_bounds__(NT, RING ? 3 : 4) k_ana(AnaArgs a) {
-  static_assert(!RING || (NS > 0 && MODE == WAVE_ITERATE),
-                "the U ring serves the size-specialised iteration kernels (full tiles)");
+// Small levels (ana_cols.cu serves the rest).
+template <int CH, int MODE, bool LEVEL1>
+__global__ void __launch_bounds__(NT, 4) k_ana(AnaArgs a) {
   extern __shared__ float2 smem2[];
   float2 *in_s = smem2;                     // [CH][A_RP][A_IP] row pairs
   float2 *lohi = in_s + CH * A_RP * A_IP;   // [A_RP][A_LP] lo, then hi
-  float *ring = reinterpret_cast<float *>(reinterpret_cast<char *>(smem2) + ring_off(CH));
-  const int n = NS ? NS : a.n, M = MS ? MS : a.M;
+  const int n = a.n, M = a.M;
   const int h = M >> 1;
   const int ntx = (h + TX - 1) / TX;
   const int kx0 = (blockIdx.x % ntx) * TX, ky0 = (blockIdx.x / ntx) * TY;
@@ -386,151 +362,19 @@ __global__ void __launch_bounds__(NT, RING ? 3 : 4) k_ana(AnaArgs a) {
   const int nsteps = (LEVEL1 ? a.K : 1) * CH;
   constexpr int LH = A_RP * A_LP;
   uint32_t keep = 0;
-  // ring variant: the detail tiles (DX, DY, HH; TY rows of TX coefficients
-  // each) of step t go to slot t mod RING_SLOTS, in 16-byte copies
-  auto ring_issue = [&](int t) {
-    if (RING && t < nsteps) {
-      const int bt = b0 + t / CH, ct = t % CH;
-      const int hh = M >> 1, hn = hh * n;
-      const float *up = a.u + ((size_t)(ct * a.L + l) * a.K + bt) * ((size_t)n * n);
-      float *slot = ring + (size_t)(t % RING_SLOTS) * ring_slot_floats();
-      for (int it = threadIdx.x; it < 3 * TY * (TX / 4); it += NT) {
-        const int sb = it / (TY * (TX / 4)), r = (it / (TX / 4)) % TY, q = it % (TX / 4);
-        const int so = sb == 0 ? hh : (sb == 1 ? hn : hn + hh);
-        cp_async16(slot + (sb * TY + r) * TX + 4 * q, up + so + (ky0 + r) * n + kx0 + 4 * q);
-      }
-    }
-    if (RING) cp_commit();
-  };
-  for (int t = 0; t < RING_AHEAD; ++t) ring_issue(t);
 #pragma unroll 1
   for (int s = 0; s < nsteps; ++s) {
     const int bb = b0 + s / CH, c = s % CH;
     float pre[4][QY];
-    if (RING) ring_issue(s + RING_AHEAD);
-    else ana_prefetch<MODE, NS, MS>(a, l, bb, c, kx0, ky0, pre);
+    ana_prefetch<MODE>(a, l, bb, c, kx0, ky0, pre);
     ana_rows_dispatch(bb + 1, in_s + c * A_RP * A_IP, lohi, lohi + LH);
-    if (RING) {
-      cp_wait<RING_AHEAD>();        // this step's tiles are in (other threads': barrier)
-      __syncthreads();
-      const float *slot = ring + (size_t)(s % RING_SLOTS) * ring_slot_floats();
-      const int kx = threadIdx.x % TX, sq = threadIdx.x / TX;
-#pragma unroll
-      for (int qq = 0; qq < QY; ++qq) {
-        const int r = QY * sq + qq;
-        pre[0][qq] = slot[(0 * TY + r) * TX + kx];
-        pre[1][qq] = slot[(1 * TY + r) * TX + kx];
-        pre[2][qq] = slot[(2 * TY + r) * TX + kx];
-        pre[3][qq] = 0.f;
-      }
-    } else {
-      __syncthreads();
-    }
+    __syncthreads();
     float cf[4][QY];
     ana_cols_dispatch(bb + 1, lohi, lohi + LH, cf);
     // dual step scale: sigma mu_l (primal, d/dgamma), sigma beta_l (d/dmu)
     const float qc = MODE == WAVE_ITERATE ? (c == 1 ? sbl : sbl * mu) : 1.f;
-    ana_emit_step<MODE, NS, MS>(a, l, bb, c, kx0, ky0, qc, cf, pre, keep);
+    ana_emit_step<MODE>(a, l, bb, c, kx0, ky0, qc, cf, pre, keep);
     __syncthreads();
-  }
-}
-
-// Level-1 analysis + dual update, pipelined: steps run chain-major (chain
-// s / K, basis s % K), and one phase holds the row pass of step s and the
-// column pass + dual update of step s - 1, with two lo/hi buffers and one
-// barrier per step, so the threads that have no row-pass item (short
-// filters) go straight to the column work.  Only z0 and one derivative
-// chain's input tile are resident (the second tile holds chain 1's input,
-// then chain 2's), and chain 0's masks of every basis stay in a 64-bit
-// register (8 bits per basis), so shared memory stays at 4 CTAs per SM.  The
-// U values of a step are requested one phase ahead.  The row and column
-// passes, the inputs and the dual update are k_ana's, so the results are
-// bit-identical.  Not the last level (J > 1).
-constexpr size_t ana_pipe_smem(int ch) {
-  return ((size_t)(ch == 3 ? 2 : 1) * A_RP * A_IP + 4 * A_RP * A_LP) * sizeof(float2);
-}
-
-template <int CH, int NS, int MS>
-__global__ void __launch_bounds__(NT, 4) k_ana_pipe(AnaArgs a) {
-  static_assert(CH == 1 || CH == 3, "one or three chains");
-  extern __shared__ float2 smem2[];
-  constexpr int TILE = A_RP * A_IP, LH = A_RP * A_LP;
-  float2 *in0 = smem2;                           // chain 0: z0
-  float2 *in1 = in0 + (CH == 3 ? TILE : 0);      // chain 1, then chain 2
-  float2 *lohi = in0 + (CH == 3 ? 2 : 1) * TILE; // [2 buffers][lo, hi]
-  const int n = NS ? NS : a.n, M = MS ? MS : a.M;
-  const int h = M >> 1;
-  const int ntx = (h + TX - 1) / TX;
-  const int kx0 = (blockIdx.x % ntx) * TX, ky0 = (blockIdx.x / ntx) * TY;
-  const int l = blockIdx.y;
-  const int K = a.K;
-  const int RP = TY + K - 1, RW = 2 * TX + 2 * K - 2;
-  const int Mm = M - 1;
-  const size_t NN = (size_t)n * n;
-  const size_t CS = (size_t)a.L * NN;
-  const DevScalars &S = a.sc[l / a.Lc];
-  const float mu = (float)S.mu;
-  const float sbl = (float)(S.sigma * (double)a.beta[l]);
-  auto zval = [&](int c, size_t pix) { return 2.f * a.xt[c * CS + pix] - a.x[c * CS + pix]; };
-  // z0 into in0 and (three chains) z0 + mu z1 into in1
-  for (int it = threadIdx.x; it < RP * RW; it += NT) {
-    const int rp = it / RW, cc = it - rp * RW;
-    const int xx = (2 * kx0 + cc) & Mm;
-    float z0[2], w1[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int yy = (2 * ky0 + 2 * rp + e) & Mm;
-      const size_t pix = (size_t)l * NN + (size_t)yy * n + xx;
-      z0[e] = zval(0, pix);
-      if (CH == 3) w1[e] = fmaf(mu, zval(1, pix), z0[e]);
-    }
-    in0[rp * A_IP + cc] = make_float2(z0[0], z0[1]);
-    if (CH == 3) in1[rp * A_IP + cc] = make_float2(w1[0], w1[1]);
-  }
-  const int nsteps = K * CH;
-  uint64_t keep = 0;
-  float pre[4][QY];
-  ana_prefetch<WAVE_ITERATE, NS, MS>(a, l, 0, 0, kx0, ky0, pre);
-  __syncthreads();
-#pragma unroll 1
-  for (int s = 0; s <= nsteps; ++s) {
-    if (CH == 3 && s == 2 * K) {
-      // chain 2's input replaces chain 1's (whose last row pass ended before
-      // the previous barrier)
-      for (int it = threadIdx.x; it < RP * RW; it += NT) {
-        const int rp = it / RW, cc = it - rp * RW;
-        const int xx = (2 * kx0 + cc) & Mm;
-        float z2[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int yy = (2 * ky0 + 2 * rp + e) & Mm;
-          z2[e] = zval(2, (size_t)l * NN + (size_t)yy * n + xx);
-        }
-        in1[rp * A_IP + cc] = make_float2(z2[0], z2[1]);
-      }
-      __syncthreads();
-    }
-    if (s < nsteps) {
-      const int c = s / K, bb = s - c * K;
-      float2 *lh = lohi + (s & 1) * 2 * LH;
-      ana_rows_dispatch(bb + 1, c == 0 ? in0 : in1, lh, lh + LH);
-    }
-    if (s >= 1) {
-      const int t = s - 1, c = t / K, bb = t - c * K;
-      const float2 *lh = lohi + (t & 1) * 2 * LH;
-      float cf[4][QY];
-      ana_cols_dispatch(bb + 1, lh, lh + LH, cf);
-      // dual step scale: sigma mu_l (primal, d/dgamma), sigma beta_l (d/dmu)
-      const float qc = c == 1 ? sbl : sbl * mu;
-      uint32_t kb = c == 0 ? 0u : (uint32_t)(keep >> (8 * bb)) & 0xffu;
-      ana_emit_step<WAVE_ITERATE, NS, MS>(a, l, bb, c, kx0, ky0, qc, cf, pre, kb);
-      if (c == 0) keep |= (uint64_t)kb << (8 * bb);
-      if (s < nsteps) {
-        const int c2 = s / K;
-        ana_prefetch<WAVE_ITERATE, NS, MS>(a, l, s - c2 * K, c2, kx0, ky0, pre);
-      }
-    }
-    if (s < nsteps) __syncthreads();
   }
 }
 
@@ -1027,51 +871,17 @@ inline double level_flops(int CH, int L, int K, int h) {
   return (double)CH * L * 32.0 * (K * (K + 1) / 2) * (double)h * h;
 }
 
-template <int CH, int MODE, bool L1, int NS = 0, int MS = 0, bool RING = false>
-cudaError_t launch_ana(const AnaArgs &a, int nblk_y, cudaStream_t st, Prof *prof) {
-  const double h = a.M >> 1, rw = MODE == WAVE_ITERATE ? 2.0 : 1.0;
-  const double in = L1 ? (double)CH * a.L * a.M * a.M * (MODE == WAVE_ITERATE ? 8.0 : 4.0)
-                       : (double)CH * a.L * a.K * a.M * a.M * 4.0;
-  const double det = (double)CH * a.L * a.K * 3.0 * h * h * 4.0 * rw;
-  const double ll = (double)CH * a.L * a.K * h * h * 4.0 * (a.last ? rw : 1.0);
-  ProfScope ps(prof, L1 ? "ana_level1_dual" : "ana_level_dual", in + det + ll,
-               level_flops(CH, a.L, L1 ? a.K : a.K, (int)h), st);
-  constexpr size_t smem = RING ? ana_smem_ring(CH) : ana_smem(CH);
+template <int CH, int MODE, bool L1>
+cudaError_t launch_ana(const AnaArgs &a, int nblk_y, cudaStream_t st) {
+  constexpr size_t smem = ana_smem(CH);
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_ana<CH, MODE, L1, NS, MS, RING>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
-  }
-  k_ana<CH, MODE, L1, NS, MS, RING><<<dim3(tiles(a.M >> 1), nblk_y), NT, smem, st>>>(a);
-  return cudaGetLastError();
-}
-
-template <int CH, int NS, int MS>
-cudaError_t launch_ana_pipe(const AnaArgs &a, int nblk_y, cudaStream_t st, Prof *prof) {
-  const double h = a.M >> 1;
-  const double in = (double)CH * a.L * a.M * a.M * 8.0;
-  const double det = (double)CH * a.L * a.K * 3.0 * h * h * 4.0 * 2.0;
-  const double ll = (double)CH * a.L * a.K * h * h * 4.0;
-  ProfScope ps(prof, "ana_level1_dual", in + det + ll, level_flops(CH, a.L, a.K, (int)h), st);
-  constexpr size_t smem = ana_pipe_smem(CH);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_ana_pipe<CH, NS, MS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_ana<CH, MODE, L1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
     attr = true;
   }
-  k_ana_pipe<CH, NS, MS><<<dim3(tiles(a.M >> 1), nblk_y), NT, smem, st>>>(a);
+  k_ana<CH, MODE, L1><<<dim3(tiles(a.M >> 1), nblk_y), NT, smem, st>>>(a);
   return cudaGetLastError();
-}
-
-// the size-specialised analysis launch, with or without the U ring
-template <int CH, int MODE, bool L1, int NS, int MS>
-cudaError_t launch_ana_sized(const AnaArgs &a, int nblk_y, bool ring, cudaStream_t st,
-                             Prof *prof) {
-  if constexpr (MODE == WAVE_ITERATE)
-    if (ring) return launch_ana<CH, MODE, L1, NS, MS, true>(a, nblk_y, st, prof);
-  return launch_ana<CH, MODE, L1, NS, MS, false>(a, nblk_y, st, prof);
 }
 
 template <int CH, int MODE, bool L1, bool PACKED>
@@ -1137,35 +947,27 @@ cudaError_t analysis_all(const WaveArgs &w, const AnaArgs &base, cudaStream_t st
     k_ana0<CH, MODE><<<grid_elem((size_t)w.L * w.n * w.n), 256, 0, st>>>(a);
     return cudaGetLastError();
   }
-  a.M = w.n;
-  a.last = (w.J == 1);
-  a.ll_out = a.last ? nullptr : w.scratch + w.lvl_off[1];
-  // the size-specialised kernels assume a level below (J > level)
-  const bool ring = w.ana_ring != 0;
   cudaError_t e = cudaSuccess;
-  bool piped = false;
-  if constexpr (MODE == WAVE_ITERATE && (CH == 1 || CH == 3)) {
-    if (w.ana_pipe && w.J > 1) {
-      piped = true;
-      e = w.n == 2048 ? launch_ana_pipe<CH, 2048, 2048>(a, w.L, st, w.prof)
-          : w.n == 1024 ? launch_ana_pipe<CH, 1024, 1024>(a, w.L, st, w.prof)
-          : w.n == 512 ? launch_ana_pipe<CH, 512, 512>(a, w.L, st, w.prof)
-                       : launch_ana_pipe<CH, 0, 0>(a, w.L, st, w.prof);
-    }
-  }
-  if (!piped) e = (w.n == 2048 && w.J > 1) ? launch_ana_sized<CH, MODE, true, 2048, 2048>(a, w.L, ring, st, w.prof)
-                  : (w.n == 1024 && w.J > 1) ? launch_ana_sized<CH, MODE, true, 1024, 1024>(a, w.L, ring, st, w.prof)
-                  : (w.n == 512 && w.J > 1) ? launch_ana_sized<CH, MODE, true, 512, 512>(a, w.L, ring, st, w.prof)
-                                            : launch_ana<CH, MODE, true>(a, w.L, st, w.prof);
-  for (int j = 2; j <= w.J && e == cudaSuccess; ++j) {
+  for (int j = 1; j <= w.J && e == cudaSuccess; ++j) {
     a.M = w.n >> (j - 1);
-    a.in = w.scratch + w.lvl_off[j - 1];
+    a.in = j == 1 ? base.in : w.scratch + w.lvl_off[j - 1];
     a.last = (j == w.J);
     a.ll_out = a.last ? nullptr : w.scratch + w.lvl_off[j];
-    if (j == 2 && w.J > 2 && w.n == 2048) e = launch_ana_sized<CH, MODE, false, 2048, 1024>(a, w.L * w.K, ring, st, w.prof);
-    else if (j == 2 && w.J > 2 && w.n == 1024) e = launch_ana_sized<CH, MODE, false, 1024, 512>(a, w.L * w.K, ring, st, w.prof);
-    else if (j == 2 && w.J > 2 && w.n == 512) e = launch_ana_sized<CH, MODE, false, 512, 256>(a, w.L * w.K, ring, st, w.prof);
-    else e = launch_ana<CH, MODE, false>(a, w.L * w.K, st, w.prof);
+    const double h = a.M >> 1, rw = MODE == WAVE_ITERATE ? 2.0 : 1.0;
+    const double in = j == 1 ? (double)CH * a.L * a.M * a.M * (MODE == WAVE_ITERATE ? 8.0 : 4.0)
+                             : (double)CH * a.L * a.K * a.M * a.M * 4.0;
+    const double det = (double)CH * a.L * a.K * 3.0 * h * h * 4.0 * rw;
+    const double ll = (double)CH * a.L * a.K * h * h * 4.0 * (a.last ? rw : 1.0);
+    ProfScope ps(w.prof, j == 1 ? "ana_level1_dual" : "ana_level_dual", in + det + ll,
+                 level_flops(CH, a.L, a.K, (int)h), st);
+    // the columns kernel's items are whole 16-byte groups (a caller's own U of
+    // the operator may start anywhere), and its tiles 64 wide: below 32
+    // coefficients a side at level 1, 64 at a coarser level, k_ana's smaller
+    // tiles win (256 x 256 x 32, three chains, level 3: 19 against 28 us)
+    const bool vec = ((reinterpret_cast<uintptr_t>(a.u) | reinterpret_cast<uintptr_t>(a.ll_out)) & 15) == 0;
+    if (a.M >= (j == 1 ? 64 : 128) && vec) e = ana_cols(a, CH, MODE == WAVE_ITERATE, j == 1, w.ana_pipe, st);
+    else if (j == 1) e = launch_ana<CH, MODE, true>(a, w.L, st);
+    else e = launch_ana<CH, MODE, false>(a, w.L * w.K, st);
   }
   return e;
 }
@@ -1193,6 +995,7 @@ cudaError_t upload_filters(const double h[8][16]) {
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_gg, gg, sizeof(gg));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_hp, hp, sizeof(hp));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_gp, gp, sizeof(gp));
+  if (e == cudaSuccess) e = upload_cols_filters(hp, gp);
   return e;
 }
 
@@ -1212,7 +1015,7 @@ cudaError_t wavelet_analysis_dual(const WaveArgs &w, const Group &gr,
                                   cudaStream_t st) {
   if (w.dict == 1 && w.J > 0) return iuwt_analysis_dual(w, gr, st);
   AnaArgs a{};
-  a.n = w.n; a.L = w.L; a.K = w.K;
+  a.n = w.n; a.L = w.L; a.K = w.K; a.masks = w.masks;
   a.Lc = w.Lc > 0 ? w.Lc : w.L;
   a.xt = gr.xt; a.x = gr.x; a.u = gr.u; a.beta = w.beta; a.sc = w.sc;
   if (gr.C == 3) return analysis_all<3, WAVE_ITERATE>(w, a, st);
