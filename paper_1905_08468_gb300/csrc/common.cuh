@@ -29,6 +29,20 @@ struct Group {
   const float *b;  // [L][n][n] H^T y of this group's data (chain 0 only)
 };
 
+// What a scan of one image finds (FP32 and integer work only).
+struct ImageStat {
+  unsigned max_bits;    // bits of the largest |x| among the finite values
+  unsigned nonfinite;   // NaN/Inf entries
+  unsigned negative;    // entries < 0
+  unsigned pad;
+};
+
+// The power of two that takes a spectrum with largest |h|^2 = m2 to a largest
+// magnitude in [1, 4); 1 for a zero spectrum, NaN for one that is not finite.
+__device__ __forceinline__ double spectrum_scale(double m2) {
+  return isfinite(m2) ? (m2 > 0.0 ? ldexp(1.0, -(ilogb(m2) >> 1)) : 1.0) : nan("");
+}
+
 __host__ __device__ inline int ilog2(int v) {
   int r = 0;
   while ((1 << r) < v) ++r;

@@ -12,9 +12,31 @@
 
 namespace muffin {
 
-template <typename C> struct Real;
-template <> struct Real<float2> { using type = float; };
-template <> struct Real<double2> { using type = double; };
+// A number as the unevaluated sum of two FP32 values, h = RN(h + l): 48 bits, at
+// the FP32 rate (Dekker, Numer. Math. 18, 1971; products by FMA).  The
+// intrinsics keep the compiler from contracting the error terms away.
+struct dd {
+  float h, l;
+};
+struct __align__(16) cdd {
+  dd x, y;
+};
+__device__ __forceinline__ dd dd_norm(float s, float e) {   // |s| >= |e|
+  const float h = __fadd_rn(s, e);
+  return dd{h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ dd operator+(dd a, dd b) {
+  const float s = __fadd_rn(a.h, b.h), v = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, v)), __fsub_rn(b.h, v));
+  return dd_norm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ dd operator-(dd a) { return dd{-a.h, -a.l}; }
+__device__ __forceinline__ dd operator-(dd a, dd b) { return a + (-b); }
+__device__ __forceinline__ dd operator*(dd a, dd b) {
+  const float p = __fmul_rn(a.h, b.h);
+  const float e = __fmaf_rn(a.h, b.h, -p);
+  return dd_norm(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, e)));
+}
 
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) {
   C r; r.x = a.x + b.x; r.y = a.y + b.y; return r;

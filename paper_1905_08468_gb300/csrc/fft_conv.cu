@@ -182,15 +182,16 @@ k_rows_inv(const float2 *__restrict__ S, float *__restrict__ g,
 }
 
 // ---------------------------------------------------------------- FP64 set-up
-__global__ void k_fft64_rows(double2 *data, int n, bool inverse,
-                             const double2 *__restrict__ tw) {
+// C: double2, or cdd (pairs of FP32 values, see fft.cuh)
+template <typename C>
+__global__ void k_fft_rows(C *data, int n, bool inverse, const C *__restrict__ tw) {
   extern __shared__ double2 sm4[];
-  double2 *a = sm4, *b = sm4 + n;
-  double2 *row = data + ((size_t)blockIdx.y * n + blockIdx.x) * n;
+  C *a = reinterpret_cast<C *>(sm4), *b = a + n;
+  C *row = data + ((size_t)blockIdx.y * n + blockIdx.x) * n;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a[i] = row[i];
   __syncthreads();
-  const double2 *r = inverse ? fft_batch<double2, true>(a, b, n, 1, tw)
-                             : fft_batch<double2, false>(a, b, n, 1, tw);
+  const C *r = inverse ? fft_batch<C, true>(a, b, n, 1, tw)
+                       : fft_batch<C, false>(a, b, n, 1, tw);
   for (int i = threadIdx.x; i < n; i += blockDim.x) row[i] = r[i];
 }
 
@@ -210,18 +211,154 @@ __global__ void k_transpose64(const double2 *__restrict__ in,
   }
 }
 
-__global__ void k_real_to_c64(const float *__restrict__ in,
-                              double2 *__restrict__ out, size_t count) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count;
-       i += (size_t)gridDim.x * blockDim.x)
-    out[i] = make_double2((double)in[i], 0.0);
+// ---- real images, two bands of a cube in one complex image
+//
+// The FP64 pipe bounds these transforms (2 operations a clock and SM against
+// 128 in FP32), so bands 2j and 2j + 1 of a cube are the real and imaginary
+// parts of one image (an odd last band rides alone): half the butterflies and
+// half the traffic of one complex image a band.  Where the result is rounded to
+// FP32 (H^T y, H^T delta), the transforms run on pairs of FP32 values (48 bits,
+// fft.cuh) instead: 1024 x 1024 x 64, a pass over the rows 2.0 -> 0.58 ms; the
+// spectra themselves (beta, |h_hat|^2) and the objective's residual stay in FP64.
+//
+// An image is scaled by a power of two (exact) to a largest magnitude in
+// [1, 2), and a band's spectrum h by one to [1, 2) or [2, 4), so that a faint
+// band keeps its own precision beside a bright one; a band with NaN/Inf enters
+// as zero and comes out as NaN, and leaves its neighbour alone.  Spectra stay
+// transposed ([kx][ky]): one transpose each way.
+
+// 2^-e of an image from its statistics: 1 for a zero image, NaN if any value is
+// not finite
+__device__ __forceinline__ double image_scale(const ImageStat &t) {
+  const float m = __uint_as_float(t.max_bits);
+  return t.nonfinite ? nan("") : (m > 0.f ? ldexp(1.0, -ilogbf(m)) : 1.0);
 }
 
-__global__ void k_mul_conj_c64(double2 *__restrict__ a,
-                               const double2 *__restrict__ h, size_t count) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count;
-       i += (size_t)gridDim.x * blockDim.x)
-    a[i] = cmulc(a[i], h[i]);
+struct Pairs {
+  int n, L, per_cube;           // side, bands per cube, pairs per cube
+  const ImageStat *stat;        // [images]
+  const double *hmax;           // [images] largest |h|^2 (not finite: h is not)
+  __device__ double scale(int img) const { return image_scale(stat[img]); }
+  __device__ double hscale(int img) const { return spectrum_scale(hmax[img]); }
+  __device__ int first(int p) const { return p / per_cube * L + 2 * (p % per_cube); }
+  __device__ bool second(int p) const { return 2 * (p % per_cube) + 1 < L; }
+};
+
+__device__ __forceinline__ void set_parts(double2 &z, double x, double y) { z = make_double2(x, y); }
+__device__ __forceinline__ void set_parts(cdd &z, double x, double y) {
+  z.x.h = (float)x; z.x.l = (float)(x - (double)z.x.h);
+  z.y.h = (float)y; z.y.l = (float)(y - (double)z.y.h);
+}
+// FP32 values times a power of two (FP32: in two factors, for its whole range)
+__device__ __forceinline__ float times_pow2(float x, double s) {
+  const int e = ilogb(s);
+  return x * ldexpf(1.f, e / 2) * ldexpf(1.f, e - e / 2);
+}
+__device__ __forceinline__ void set_input(double2 &z, float x, double sx, float y, double sy) {
+  z = make_double2(sx * (double)x, sy * (double)y);
+}
+__device__ __forceinline__ void set_input(cdd &z, float x, double sx, float y, double sy) {
+  z = cdd{{sx != 0.0 ? times_pow2(x, sx) : 0.f, 0.f}, {sy != 0.0 ? times_pow2(y, sy) : 0.f, 0.f}};
+}
+__device__ __forceinline__ float to_float(double v, double c) { return (float)(c * v); }
+__device__ __forceinline__ float to_float(dd v, double c) {   // c a power of two or NaN
+  return c == c ? times_pow2(v.h, c) : __int_as_float(0x7fc00000);
+}
+
+// forward transform along x of the packed rows: grid (n, pairs)
+template <typename C>
+__global__ void k_rows_real(const float *__restrict__ x, C *__restrict__ out, Pairs P,
+                            const C *__restrict__ tw) {
+  extern __shared__ double2 sm4[];
+  const int n = P.n, p = blockIdx.y, ia = P.first(p);
+  const bool two = P.second(p);
+  C *a = reinterpret_cast<C *>(sm4), *b = a + n;
+  const float *xa = x + ((size_t)ia * n + blockIdx.x) * n, *xb = xa + (size_t)n * n;
+  const double sa = P.scale(ia), sb = two ? P.scale(ia + 1) : 0.0;
+  const bool oka = sa == sa, okb = two && sb == sb;
+  for (int i = threadIdx.x; i < n; i += blockDim.x)
+    set_input(a[i], oka ? xa[i] : 0.f, oka ? sa : 0.0, okb ? xb[i] : 0.f, okb ? sb : 0.0);
+  __syncthreads();
+  const C *r = fft_batch<C, false>(a, b, n, 1, tw);
+  C *row = out + ((size_t)p * n + blockIdx.x) * n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) row[i] = r[i];
+}
+
+// inverse transform along x of the packed rows and the two real images
+// out = (float)(c / scales * part): grid (n, pairs)
+template <typename C>
+__global__ void k_rows_out(const C *__restrict__ w, float *__restrict__ out, Pairs P,
+                           double c, const C *__restrict__ tw) {
+  extern __shared__ double2 sm4[];
+  const int n = P.n, p = blockIdx.y, ia = P.first(p);
+  C *a = reinterpret_cast<C *>(sm4), *b = a + n;
+  const C *row = w + ((size_t)p * n + blockIdx.x) * n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) a[i] = row[i];
+  __syncthreads();
+  const C *r = fft_batch<C, true>(a, b, n, 1, tw);
+  float *oa = out + ((size_t)ia * n + blockIdx.x) * n, *ob = oa + (size_t)n * n;
+  const bool two = P.second(p);
+  const double ca = c / (P.scale(ia) * P.hscale(ia));
+  const double cb = two ? c / (P.scale(ia + 1) * P.hscale(ia + 1)) : 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    oa[i] = to_float(r[i].x, ca);
+    if (two) ob[i] = to_float(r[i].y, cb);
+  }
+}
+
+__device__ __forceinline__ double half_of(double v) { return 0.5 * v; }
+__device__ __forceinline__ dd half_of(dd v) { return dd{0.5f * v.h, 0.5f * v.l}; }
+
+// the spectra A, B of the packed images at k, from Z[k] and Z[-k]
+template <typename C>
+__device__ __forceinline__ void pair_split(const C &z, const C &m, C &A, C &B) {
+  A.x = half_of(z.x + m.x); A.y = half_of(z.y - m.y);
+  B.x = half_of(z.y + m.y); B.y = half_of(m.x - z.x);
+}
+
+// spectra of every band from the packed ones: grid (n, pairs), row kx
+__global__ void k_pair_unpack(const double2 *__restrict__ z, double2 *__restrict__ hh, Pairs P) {
+  const int n = P.n, p = blockIdx.y, ia = P.first(p), kx = blockIdx.x;
+  const size_t N = (size_t)n * n, row = (size_t)kx * n;
+  const double2 *zr = z + p * N + row, *zm = z + p * N + (size_t)((n - kx) & (n - 1)) * n;
+  const bool two = P.second(p);
+  const double ra = 1.0 / P.scale(ia), rb = two ? 1.0 / P.scale(ia + 1) : 0.0;
+  double2 *ha = hh + ia * N + row, *hb = ha + N;
+  for (int ky = threadIdx.x; ky < n; ky += blockDim.x) {
+    double2 A, B;
+    pair_split(zr[ky], zm[(n - ky) & (n - 1)], A, B);
+    ha[ky] = make_double2(ra * A.x, ra * A.y);
+    if (two) hb[ky] = make_double2(rb * B.x, rb * B.y);
+  }
+}
+
+// packed spectra times every band's own scaled h (CJ: its conjugate), in place:
+// grid (n / 2 + 1, pairs), rows kx and -kx; a thread takes k and -k (the images
+// are real, so -k holds the conjugates)
+template <typename C, bool CJ>
+__global__ void k_pair_mul(C *__restrict__ z, const double2 *__restrict__ hh, Pairs P) {
+  const int n = P.n, p = blockIdx.y, ia = P.first(p), kx = blockIdx.x, mx = (n - kx) & (n - 1);
+  const size_t N = (size_t)n * n, row = (size_t)kx * n;
+  C *zr = z + p * N + row, *zm = z + p * N + (size_t)mx * n;
+  const double2 *ha = hh + ia * N + row, *hb = ha + N;
+  const bool two = P.second(p);
+  const double sa = P.hscale(ia), sb = two ? P.hscale(ia + 1) : 0.0;
+  const bool oka = sa == sa, okb = two && sb == sb;
+  for (int ky = threadIdx.x; ky < n; ky += blockDim.x) {
+    const int my = (n - ky) & (n - 1);
+    if (mx == kx && my < ky) continue;
+    C A, B, h;
+    pair_split(zr[ky], zm[my], A, B);
+    set_parts(h, oka ? sa * ha[ky].x : 0.0, oka ? sa * ha[ky].y : 0.0);
+    A = CJ ? cmulc(A, h) : cmul(A, h);
+    set_parts(h, okb ? sb * hb[ky].x : 0.0, okb ? sb * hb[ky].y : 0.0);
+    B = CJ ? cmulc(B, h) : cmul(B, h);
+    C w, v;
+    w.x = A.x + B.y; w.y = B.x - A.y;              // conj A + i conj B
+    v.x = A.x - B.y; v.y = A.y + B.x;              // A + i B (k == -k: the same real parts)
+    zm[my] = w;
+    zr[ky] = v;
+  }
 }
 
 __global__ void k_c64_real_to_f32(const double2 *__restrict__ in,
@@ -232,20 +369,30 @@ __global__ void k_c64_real_to_f32(const double2 *__restrict__ in,
     out[i] = (float)(in[i].x * scale);
 }
 
-__global__ void k_make_kspec(const double2 *__restrict__ hh,
-                             float *__restrict__ kspec, double scale, int n,
-                             int L) {
-  const int nh = (n >> 1) + 1;
-  const size_t total = (size_t)L * nh * n;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int ky = (int)(i % n);
-    const size_t r = i / n;
-    const int kx = (int)(r % nh);
-    const int l = (int)(r / nh);
-    const double2 h = hh[((size_t)l * n + ky) * n + kx];
-    kspec[i] = (float)((h.x * h.x + h.y * h.y) * scale);
+// grid (n / 2 + 1, L); max_bits[l]: the largest |hh|^2 of the band (bits of a
+// double >= 0, which order as integers, and above them NaN; the other half of a
+// spectrum holds the conjugates)
+__global__ void k_make_kspec(const double2 *__restrict__ hh, float *__restrict__ kspec,
+                             double scale, int n, unsigned long long *max_bits) {
+  const int l = blockIdx.y, kx = blockIdx.x;
+  const double2 *h = hh + ((size_t)l * n + kx) * n;
+  float *k = kspec + ((size_t)l * ((n >> 1) + 1) + kx) * n;
+  unsigned long long m = 0;
+  for (int ky = threadIdx.x; ky < n; ky += blockDim.x) {
+    const double v = h[ky].x * h[ky].x + h[ky].y * h[ky].y;
+    m = max(m, (unsigned long long)__double_as_longlong(fabs(v)));
+    k[ky] = (float)(v * scale);
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
+    m = m > t ? m : t;
+  }
+  if ((threadIdx.x & 31) == 0) atomicMax(max_bits + l, m);
+}
+
+template <typename F>
+void allow_smem(F *k) {
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
 inline int grid_for(size_t count) {
@@ -341,29 +488,85 @@ cudaError_t fft2d_c64(double2 *data, double2 *tmp, int n, int nimg,
                       bool inverse, const double2 *tw64, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_fft64_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    allow_smem(k_fft_rows<double2>);
     attr = true;
   }
   const size_t sm = (size_t)2 * n * sizeof(double2);
   const int thr = n < 256 ? (n < 32 ? 32 : n) : 256;
   dim3 tg((n + 31) / 32, (n + 31) / 32, nimg), tb(32, 8);
-  k_fft64_rows<<<dim3(n, nimg), thr, sm, st>>>(data, n, inverse, tw64);
+  k_fft_rows<double2><<<dim3(n, nimg), thr, sm, st>>>(data, n, inverse, tw64);
   k_transpose64<<<tg, tb, 0, st>>>(data, tmp, n);
-  k_fft64_rows<<<dim3(n, nimg), thr, sm, st>>>(tmp, n, inverse, tw64);
+  k_fft_rows<double2><<<dim3(n, nimg), thr, sm, st>>>(tmp, n, inverse, tw64);
   k_transpose64<<<tg, tb, 0, st>>>(tmp, data, n);
   return cudaGetLastError();
 }
 
-cudaError_t real_to_c64(const float *in, double2 *out, size_t count,
-                        cudaStream_t st) {
-  k_real_to_c64<<<grid_for(count), 256, 0, st>>>(in, out, count);
+namespace {
+int row_threads(int n) { return n < 256 ? (n < 32 ? 32 : n) : 256; }
+
+// z (pairs) = spectra of the packed images, [kx][ky]
+template <typename C>
+cudaError_t pair_forward(const float *x, const Pairs &P, int np, C *z, C *tmp, const C *tw,
+                         cudaStream_t st) {
+  const int n = P.n;
+  const size_t sm = (size_t)2 * n * sizeof(C);
+  allow_smem(k_rows_real<C>);
+  allow_smem(k_fft_rows<C>);
+  k_rows_real<C><<<dim3(n, np), row_threads(n), sm, st>>>(x, tmp, P, tw);
+  k_transpose64<<<dim3((n + 31) / 32, (n + 31) / 32, np), dim3(32, 8), 0, st>>>(
+      reinterpret_cast<double2 *>(tmp), reinterpret_cast<double2 *>(z), n);
+  k_fft_rows<C><<<dim3(n, np), row_threads(n), sm, st>>>(z, n, false, tw);
   return cudaGetLastError();
 }
 
-cudaError_t mul_conj_c64(double2 *a, const double2 *h, size_t count,
-                         cudaStream_t st) {
-  k_mul_conj_c64<<<grid_for(count), 256, 0, st>>>(a, h, count);
+template <typename C, bool CJ>
+cudaError_t pair_convolve(const float *x, const Pairs &P, int np, const double2 *hh, C *z, C *tmp,
+                          double c, float *out, const C *tw, cudaStream_t st) {
+  cudaError_t e = pair_forward<C>(x, P, np, z, tmp, tw, st);
+  if (e != cudaSuccess) return e;
+  const int n = P.n;
+  const size_t sm = (size_t)2 * n * sizeof(C);
+  const dim3 rows(n, np);
+  k_pair_mul<C, CJ><<<dim3((n >> 1) + 1, np), row_threads(n), 0, st>>>(z, hh, P);
+  k_fft_rows<C><<<rows, row_threads(n), sm, st>>>(z, n, true, tw);
+  k_transpose64<<<dim3((n + 31) / 32, (n + 31) / 32, np), dim3(32, 8), 0, st>>>(
+      reinterpret_cast<double2 *>(z), reinterpret_cast<double2 *>(tmp), n);
+  if (out) {
+    allow_smem(k_rows_out<C>);
+    k_rows_out<C><<<rows, row_threads(n), sm, st>>>(tmp, out, P, c, tw);
+  } else {
+    k_fft_rows<C><<<rows, row_threads(n), sm, st>>>(tmp, n, true, tw);
+  }
   return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t spectra_real(const float *x, const ImageStat *stat, int n, int L, int nimg,
+                         double2 *hh, double2 *z, double2 *tmp, const double2 *tw64,
+                         cudaStream_t st) {
+  const Pairs P{n, L, (L + 1) / 2, stat, nullptr};
+  const int np = nimg / L * P.per_cube;
+  cudaError_t e = pair_forward<double2>(x, P, np, z, tmp, tw64, st);
+  if (e != cudaSuccess) return e;
+  k_pair_unpack<<<dim3(n, np), row_threads(n), 0, st>>>(z, hh, P);
+  return cudaGetLastError();
+}
+
+cudaError_t adjoint_real(const float *x, const ImageStat *stat, const double2 *hh,
+                         const double *hmax, int n, int L, int nimg, double2 *z, double2 *tmp,
+                         float *out, const float4 *twdd, cudaStream_t st) {
+  const Pairs P{n, L, (L + 1) / 2, stat, hmax};
+  return pair_convolve<cdd, true>(x, P, nimg / L * P.per_cube, hh, reinterpret_cast<cdd *>(z),
+                                  reinterpret_cast<cdd *>(tmp), 1.0 / ((double)n * n), out,
+                                  reinterpret_cast<const cdd *>(twdd), st);
+}
+
+cudaError_t convolve_real(const float *x, const ImageStat *stat, const double2 *hh,
+                          const double *hmax, int n, int L, int nimg, double2 *z, double2 *tmp,
+                          const double2 *tw64, cudaStream_t st) {
+  const Pairs P{n, L, (L + 1) / 2, stat, hmax};
+  return pair_convolve<double2, false>(x, P, nimg / L * P.per_cube, hh, z, tmp, 0.0, nullptr,
+                                       tw64, st);
 }
 
 cudaError_t c64_real_to_f32(const double2 *in, float *out, double scale,
@@ -373,9 +576,11 @@ cudaError_t c64_real_to_f32(const double2 *in, float *out, double scale,
 }
 
 cudaError_t make_kspec(const double2 *hh, float *kspec, double scale, int n,
-                       int L, cudaStream_t st) {
-  const size_t total = (size_t)L * ((n >> 1) + 1) * n;
-  k_make_kspec<<<grid_for(total), 256, 0, st>>>(hh, kspec, scale, n, L);
+                       int L, double *hmax, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(hmax, 0, (size_t)L * sizeof(double), st);
+  if (e != cudaSuccess) return e;
+  k_make_kspec<<<dim3((n >> 1) + 1, L), row_threads(n), 0, st>>>(
+      hh, kspec, scale, n, reinterpret_cast<unsigned long long *>(hmax));
   return cudaGetLastError();
 }
 

@@ -111,22 +111,32 @@ void fft32_tables(int n, float2 *tab, int radix = 16);
 // In-place 2D DFT of nimg complex n x n images; inverse is unnormalised.
 cudaError_t fft2d_c64(double2 *data, double2 *tmp, int n, int nimg, bool inverse,
                       const double2 *tw64, cudaStream_t st);
-cudaError_t real_to_c64(const float *in, double2 *out, size_t count,
-                        cudaStream_t st);
-// a *= conj(h) elementwise (count elements)
-cudaError_t mul_conj_c64(double2 *a, const double2 *h, size_t count,
+// FP64 spectra of nimg real images (whole cubes of L bands), two bands of a cube
+// in one complex image: hh [nimg][kx][ky].  stat: image_stats of x; z and tmp:
+// ceil(L / 2) n^2 complex a cube each.
+cudaError_t spectra_real(const float *x, const ImageStat *stat, int n, int L, int nimg,
+                         double2 *hh, double2 *z, double2 *tmp, const double2 *tw64,
                          cudaStream_t st);
+// out = H^T x of nimg real images (whole cubes) on pairs of FP32 values (48
+// bits), rounded to FP32.  hmax [nimg]: make_kspec's; twdd [n]: the twiddles as
+// (hi, lo) of the cosine and of the sine.
+cudaError_t adjoint_real(const float *x, const ImageStat *stat, const double2 *hh,
+                         const double *hmax, int n, int L, int nimg, double2 *z, double2 *tmp,
+                         float *out, const float4 *twdd, cudaStream_t st);
+// FP64 H x, unnormalised, left in tmp: band 2j (2j + 1) of a cube in the real
+// (imaginary) part of its pair j, times the powers of two of band and spectrum.
+cudaError_t convolve_real(const float *x, const ImageStat *stat, const double2 *hh,
+                          const double *hmax, int n, int L, int nimg, double2 *z, double2 *tmp,
+                          const double2 *tw64, cudaStream_t st);
 // out = (float)(scale * in.x)
 cudaError_t c64_real_to_f32(const double2 *in, float *out, double scale,
                             size_t count, cudaStream_t st);
-// kspec[l][kx][ky] = |hh[l][ky][kx]|^2 * scale for kx < n/2+1
+// kspec[l][kx][ky] = |hh[l][kx][ky]|^2 * scale for kx < n/2+1; hmax[l] = the
+// largest |hh[l]|^2 (NaN if any is)
 cudaError_t make_kspec(const double2 *hh, float *kspec, double scale, int n,
-                       int L, cudaStream_t st);
+                       int L, double *hmax, cudaStream_t st);
 
 // ------------------------------------------------------------ reductions (reduce.cu)
-// out[0] = max |hh|^2 over count complex values (FP64); scratch >= 1024 doubles
-cudaError_t max_abs2_c64(const double2 *hh, size_t count, double *scratch,
-                         double *out, cudaStream_t st);
 // per-band sum of squares: out[l] = sum y[l]^2 (FP64)
 cudaError_t band_sumsq(const float *y, int L, size_t per_band, double *out,
                        cudaStream_t st);
@@ -186,15 +196,17 @@ size_t monitor_scratch_doubles(int L);
 // of NaN/Inf entries of x} over the N values of band l (FP64)
 cudaError_t mon_state(const float *x, const float *xo, int L, size_t N, double *scratch,
                       double *out, cudaStream_t st);
-// out[l] = sum_i (scale * w[l][i].x - y[l][i])^2 (FP64)
-cudaError_t mon_resid2(const double2 *w, const float *y, double scale, int L, size_t N,
-                       double *scratch, double *out, cudaStream_t st);
+// stat[l] of L images of N values
+cudaError_t image_stats(const float *x, int L, size_t N, ImageStat *stat, cudaStream_t st);
+// out[l] = sum_i (c w / scales - y[l][i])^2 (FP64), w band l's part of the packed
+// images of convolve_real (Lc bands a cube, its stat and hmax)
+cudaError_t mon_resid2(const double2 *w, const ImageStat *stat, const double *hmax, const float *y,
+                       double c, int L, int Lc, size_t N, double *scratch, double *out,
+                       cudaStream_t st);
 // out[l] = sum_i a_i |u[l][i]| over per_band values, a_i = alpha[(l / Lc) N + i mod N]
 // (or 1 when alpha is NULL)
 cudaError_t mon_abs(const float *u, int L, size_t per_band, const float *alpha, int Lc,
                     size_t N, double *scratch, double *out, cudaStream_t st);
-// a *= h elementwise (complex FP64)
-cudaError_t mul_c64(double2 *a, const double2 *h, size_t count, cudaStream_t st);
 // z = 2 xt - x (the spectral step's input, Alg. 2 eq. vt)
 cudaError_t twice_minus(const float *xt, const float *x, float *z, size_t count,
                         cudaStream_t st);

@@ -37,8 +37,7 @@ namespace {
 
 thread_local std::string g_err = "no error";
 
-// reduction scratch layout (doubles): [0] result, [16, 16+1024) max partials;
-// band sums use [0, 65 Lt); ADA-PT partials start at kRedSure + 65 Lt.
+// reduction scratch layout (doubles): band sums use [0, 65 Lt); ADA-PT partials start at kRedSure + 65 Lt.
 constexpr size_t kRedSure = 1040;
 
 // round-to-nearest (ties away) to the 10-bit TF32 mantissa
@@ -162,28 +161,51 @@ muffin_status store(muffin_plan P, const float *src, float *dst, size_t count) {
   return MUFFIN_OK;
 }
 
-// NaN/Inf scan of an input already copied to the device (nimg images of N
-// pixels); synchronises the work stream
-muffin_status scan_input(muffin_plan P, const float *d, int nimg, const char *what) {
-  double *o = P->mon + 54 * (size_t)P->Lt;
-  CK(mon_state(d, nullptr, nimg, P->N, P->mon, o, P->ws));
-  std::vector<double> h(3 * (size_t)nimg);
-  CK(cudaMemcpyAsync(h.data(), o, h.size() * sizeof(double), cudaMemcpyDeviceToHost, P->ws));
+// statistics of an array on the device (nimg images of N pixels), to P->stat
+// and to the host; synchronises the work stream
+muffin_status image_scan(muffin_plan P, const float *d, int nimg, std::vector<ImageStat> &h) {
+  CK(image_stats(d, nimg, P->N, P->stat, P->ws));
+  h.resize((size_t)nimg);
+  CK(cudaMemcpyAsync(h.data(), P->stat, h.size() * sizeof(ImageStat), cudaMemcpyDeviceToHost,
+                     P->ws));
   CK(cudaStreamSynchronize(P->ws));
+  return MUFFIN_OK;
+}
+
+// NaN/Inf scan of an input already copied to the device; leaves its image
+// statistics in P->stat
+muffin_status scan_input(muffin_plan P, const float *d, int nimg, const char *what) {
+  std::vector<ImageStat> h;
+  muffin_status s = image_scan(P, d, nimg, h);
+  if (s != MUFFIN_OK) return s;
   double bad = 0;
-  for (int l = 0; l < nimg; ++l) bad += h[3 * (size_t)l + 2];
+  for (const ImageStat &t : h) bad += t.nonfinite;
   if (bad > 0) return fail(MUFFIN_ENUMERIC, "%s has %.0f NaN/Inf entries", what, bad);
   return MUFFIN_OK;
 }
 
-// H^T y (unnormalised, FP64) for `nimg` bands of y already on the device
-muffin_status adjoint_fp64(muffin_plan P, const float *y_dev, const double2 *hh,
-                           int nimg, double2 *w, double2 *tmp) {
-  const size_t cnt = (size_t)nimg * P->N;
-  CK(real_to_c64(y_dev, w, cnt, P->ws));
-  CK(fft2d_c64(w, tmp, P->n, nimg, false, P->tw64, P->ws));
-  CK(mul_conj_c64(w, hh, cnt, P->ws));
-  CK(fft2d_c64(w, tmp, P->n, nimg, true, P->tw64, P->ws));
+// out = H^T y for the bands of the cubes from c0 on, y on the device with its
+// statistics in P->stat; w and tmp as for spectra_real
+muffin_status adjoint(muffin_plan P, const float *y_dev, int c0, int nimg, double2 *w,
+                      double2 *tmp, float *out) {
+  CK(adjoint_real(y_dev, P->stat, P->hhat + (size_t)c0 * P->NLc, P->hmax + (size_t)c0 * P->L, P->n,
+                  P->L, nimg, w, tmp, out, P->twdd, P->ws));
+  return MUFFIN_OK;
+}
+
+// beta = the largest |h_hat|^2 of the cubes [c0, c1), from make_kspec (a band that
+// is not a number is passed over here; it shows in the results)
+muffin_status read_lipschitz(muffin_plan P, int c0, int c1, const char *what) {
+  std::vector<double> m((size_t)(c1 - c0) * P->L);
+  CK(cudaMemcpyAsync(m.data(), P->hmax + (size_t)c0 * P->L, m.size() * sizeof(double),
+                     cudaMemcpyDeviceToHost, P->ws));
+  CK(cudaStreamSynchronize(P->ws));
+  for (int c = c0; c < c1; ++c) {
+    double lip = 0;
+    for (int l = 0; l < P->L; ++l) lip = std::fmax(lip, m[(size_t)(c - c0) * P->L + l]);
+    if (!(lip > 0) || !std::isfinite(lip)) return fail(MUFFIN_EINVAL, what, c, lip);
+    P->lips[c] = lip;
+  }
   return MUFFIN_OK;
 }
 
@@ -381,6 +403,9 @@ muffin_status plan_alloc_init(muffin_plan P, const float *alpha, const float *be
   CK(cudaMemsetAsync(P->kerr, 0, sizeof(int), P->ws));
   CK(P->alloc(&P->dred, kRedSure + 65 * (size_t)Lt + 6 * (size_t)(Lt > 4096 ? Lt : 4096)));
   CK(P->alloc(&P->wband, (size_t)Lt));
+  CK(P->alloc(&P->stat, (size_t)Lt));
+  CK(P->alloc(&P->hmax, (size_t)Lt));
+  CK(P->alloc(&P->twdd, (size_t)n));
   CK(P->alloc(&P->mon, monitor_scratch_doubles(Lt)));
   CK(P->alloc(&P->S, (size_t)P->Cmax * Lt * nh * n));
   size_t off = 0;
@@ -423,6 +448,12 @@ muffin_status plan_alloc_init(muffin_plan P, const float *alpha, const float *be
     const double a = -2.0 * pi * k / n;
     t64[k] = make_double2(std::cos(a), std::sin(a));
   }
+  std::vector<float4> tdd(n);      // the same as pairs of FP32 values
+  for (int k = 0; k < n; ++k) {
+    const float ch = (float)t64[k].x, sh = (float)t64[k].y;
+    tdd[k] = make_float4(ch, (float)(t64[k].x - ch), sh, (float)(t64[k].y - sh));
+  }
+  CK(cudaMemcpyAsync(P->twdd, tdd.data(), n * sizeof(float4), cudaMemcpyHostToDevice, P->ws));
   std::vector<float2> t32((size_t)P->tw_len16 + fft32_table_len(n, 8));
   fft32_tables(n, t32.data(), 16);
   fft32_tables(n, t32.data() + P->tw_len16, 8);
@@ -541,7 +572,7 @@ struct MonOut {
 };
 
 // FP64 monitor of a cube of iterates x (device, [B][L][n][n]) against the
-// previous iterates xo (NULL: scan x only); with y (device dirty cubes) also
+// previous iterates xo (NULL: no change reported); with y (device dirty cubes) also
 // the objective (Eqs. probopt, RegAll) at x with per-cube (mu, gamma):
 // the residual y - H x from an FP64 convolution (the plan's FP64 spectra),
 // ||W_s x_l||_1 and ||W_lambda x^n||_1 from the FP32 transforms, all sums
@@ -554,15 +585,14 @@ muffin_status monitor_eval(muffin_plan P, const float *x, const float *xo, const
   double *part = P->mon;
   double *o_state = part + 48 * (size_t)Lt, *o_res = o_state + 3 * (size_t)Lt;
   double *o_u = o_res + Lt, *o_v = o_u + Lt;
-  CK(mon_state(x, xo, Lt, N, part, o_state, P->ws));
+  if (xo) CK(mon_state(x, xo, Lt, N, part, o_state, P->ws));
+  else CK(cudaMemsetAsync(o_state, 0, 3 * (size_t)Lt * sizeof(double), P->ws));
   if (y) {
     muffin_status s = ensure_op_buffers(P);
     if (s != MUFFIN_OK) return s;
-    CK(real_to_c64(x, P->w64a, P->NL, P->ws));
-    CK(fft2d_c64(P->w64a, P->w64b, P->n, Lt, false, P->tw64, P->ws));
-    CK(mul_c64(P->w64a, P->hhat, P->NL, P->ws));
-    CK(fft2d_c64(P->w64a, P->w64b, P->n, Lt, true, P->tw64, P->ws));
-    CK(mon_resid2(P->w64a, y, 1.0 / (double)N, Lt, N, part, o_res, P->ws));
+    CK(image_stats(x, Lt, N, P->stat, P->ws));
+    CK(convolve_real(x, P->stat, P->hhat, P->hmax, P->n, L, Lt, P->w64a, P->w64b, P->tw64, P->ws));
+    CK(mon_resid2(P->w64b, P->stat, P->hmax, y, 1.0 / (double)N, Lt, L, N, part, o_res, P->ws));
     CK(wavelet_analysis_op(P->wave(1), x, P->op_out, P->ws));
     CK(mon_abs(P->op_out, Lt, (size_t)P->K * N, nullptr, L, N, part, o_u, P->ws));
     CK(dct_op(P->dct(1), x, P->op_out, 0, P->ws));
@@ -627,14 +657,15 @@ muffin_status monitor_check(muffin_plan P, int k, const std::vector<double> &mu,
 
 // end-of-call scan of the restored cube for NaN/Inf
 muffin_status final_scan(muffin_plan P, int k) {
-  MonOut r;
-  std::vector<double> z(P->B, 0.0);
-  muffin_status s = monitor_eval(P, P->grp[0].x, nullptr, nullptr, z, z, r);
+  std::vector<ImageStat> h;
+  muffin_status s = image_scan(P, P->grp[0].x, P->Lt, h);
   if (s != MUFFIN_OK) return s;
-  if (r.nonfinite_total > 0) {
+  long long bad = 0;
+  for (const ImageStat &t : h) bad += t.nonfinite;
+  if (bad > 0) {
     P->have_state = P->have_sure_state = false;
     return fail(MUFFIN_ENUMERIC, "%lld NaN/Inf entries in X after %d iterations",
-                r.nonfinite_total, k);
+                bad, k);
   }
   return MUFFIN_OK;
 }
@@ -698,21 +729,13 @@ muffin_status load_psf(muffin_plan P, int b0, int b1, const float *psf) {
   muffin_status s = fetch(P, psf, P->stage_a + off, cnt);
   if (s != MUFFIN_OK) return s;
   double2 *hh = P->hhat + off;
-  CK(real_to_c64(P->stage_a + off, hh, cnt, P->ws));
-  CK(fft2d_c64(hh, P->w64a + off, P->n, nimg, false, P->tw64, P->ws));
+  CK(image_stats(P->stage_a + off, nimg, P->N, P->stat, P->ws));
+  CK(spectra_real(P->stage_a + off, P->stat, P->n, P->L, nimg, hh, P->w64a + off, P->w64b + off,
+                  P->tw64, P->ws));
   const int nh = P->n / 2 + 1;
   CK(make_kspec(hh, P->kspec + (size_t)b0 * P->L * nh * P->n, 1.0 / ((double)P->n * P->n),
-                P->n, nimg, P->ws));
-  for (int c = b0; c < b1; ++c) {
-    CK(max_abs2_c64(P->hhat + (size_t)c * P->NLc, P->NLc, P->dred + 16, P->dred, P->ws));
-    double lip = 0;
-    CK(cudaMemcpyAsync(&lip, P->dred, sizeof(double), cudaMemcpyDeviceToHost, P->ws));
-    CK(cudaStreamSynchronize(P->ws));
-    if (!(lip > 0) || !std::isfinite(lip))
-      return fail(MUFFIN_EINVAL, "PSF spectrum of cube %d is zero or not finite (beta=%g)", c, lip);
-    P->lips[c] = lip;
-  }
-  return MUFFIN_OK;
+                P->n, nimg, P->hmax + (size_t)b0 * P->L, P->ws));
+  return read_lipschitz(P, b0, b1, "PSF spectrum of cube %d is zero or not finite (beta=%g)");
 }
 
 muffin_status load_dirty(muffin_plan P, int b0, int b1, const float *dirty) {
@@ -722,10 +745,8 @@ muffin_status load_dirty(muffin_plan P, int b0, int b1, const float *dirty) {
   muffin_status s = fetch(P, dirty, P->stage_a + off, cnt);
   if (s == MUFFIN_OK) s = scan_input(P, P->stage_a + off, (b1 - b0) * P->L, "the dirty cube");
   if (s != MUFFIN_OK) return s;
-  s = adjoint_fp64(P, P->stage_a + off, P->hhat + off, (b1 - b0) * P->L, P->w64a + off,
-                   P->w64b + off);
+  s = adjoint(P, P->stage_a + off, b0, (b1 - b0) * P->L, P->w64a + off, P->w64b + off, P->b + off);
   if (s != MUFFIN_OK) return s;
-  CK(c64_real_to_f32(P->w64a + off, P->b + off, 1.0 / ((double)P->n * P->n), cnt, P->ws));
   if (P->ydev) {
     CK(cudaMemcpyAsync(P->ydev + off, P->stage_a + off, cnt * sizeof(float),
                        cudaMemcpyDeviceToDevice, P->ws));
@@ -814,13 +835,13 @@ size_t estimate_bytes(const muffin_params *p) {
     for (int j = 1; j < p->levels; ++j) ll += C * Lt * K * (n >> j) * (n >> j);
   size_t b = 3 * NL * 16 + Lt * nh * n * 4 + (size_t)(fft32_table_len((int)n, 16) + fft32_table_len((int)n, 8)) * 8 + n * 16 +
              4 * Lp * Lp * 4 + (size_t)dct_fold_table_len((int)L) * 4 + B * N * 4 + Lt * 4 + B * sizeof(DevScalars) + B * 32 + 4 + 4 +
-             (kRedSure + 65 * Lt + 6 * (Lt > 4096 ? Lt : 4096)) * 8 + Lt * 8 +
+             (kRedSure + 65 * Lt + 6 * (Lt > 4096 ? Lt : 4096)) * 8 + Lt * 8 + Lt * sizeof(ImageStat) + Lt * 8 + n * 16 +
              C * Lt * nh * n * 8 + (ll ? ll : 1) * 4 + 3 * NL * 4 +
              C * NL * (5 + K) * 4;
   if (p->sure) b += 3 * NL * (5 + K) * 4 + 2 * NL * 4 + C * Lt * nh * n * 8 + (ll ? ll : 1) * 4;
   b += monitor_scratch_doubles((int)Lt) * 8;
   if (spectral_f32(p)) b += (size_t)dct_f32_table_len((int)L) * 8 + 16;
-  return b + (p->sure ? 41 : 31) * 16;   // 16 bytes of slack per allocation
+  return b + (p->sure ? 44 : 34) * 16;   // 16 bytes of slack per allocation
 }
 
 muffin_status create(const muffin_params *p, const float *psf, const float *alpha,
@@ -948,16 +969,9 @@ muffin_status muffin_plan_load_visibilities(muffin_plan P, const float *vis,
     const std::string msg = muffin_last_error();
     return fail(MUFFIN_EINVAL, "%s", msg.c_str());
   }
-  CK(make_kspec(P->hhat, P->kspec, 1.0 / ((double)P->n * P->n), P->n, nimg, P->ws));
-  for (int c = 0; c < P->B; ++c) {
-    CK(max_abs2_c64(P->hhat + (size_t)c * P->NLc, P->NLc, P->dred + 16, P->dred, P->ws));
-    double lip = 0;
-    CK(cudaMemcpyAsync(&lip, P->dred, sizeof(double), cudaMemcpyDeviceToHost, P->ws));
-    CK(cudaStreamSynchronize(P->ws));
-    if (!(lip > 0) || !std::isfinite(lip))
-      return fail(MUFFIN_EINVAL, "the visibility weights of cube %d are all zero", c);
-    P->lips[c] = lip;
-  }
+  CK(make_kspec(P->hhat, P->kspec, 1.0 / ((double)P->n * P->n), P->n, nimg, P->hmax, P->ws));
+  s = read_lipschitz(P, 0, P->B, "the visibility weights of cube %d are all zero");
+  if (s != MUFFIN_OK) return s;
   // visibilities (re, im pairs) -> b = Re U^H D = Re(unnormalised inverse DFT of D) / n
   float *vf = reinterpret_cast<float *>(P->w64b);   // 2 cnt floats fit in cnt double2
   const cudaMemcpyKind k = is_device_ptr(vis) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
@@ -1095,18 +1109,16 @@ muffin_status muffin_sure_tune(muffin_plan P, const float *dirty,
   muffin_status s = pi::enter(P);
   if (s != MUFFIN_OK) return s;
   const size_t NL = P->NL;
-  const double scale = 1.0 / ((double)P->n * P->n);
   if (!warm) {
-    // H^T y and H^T delta in FP64; b_bar = H^T y + eps H^T delta
+    // H^T y and H^T delta; b_bar = H^T y + eps H^T delta
     s = pi::load_dirty(P, 0, B, dirty);
     if (s != MUFFIN_OK) return s;
     P->have_b = true;
     s = fetch(P, delta, P->stage_b, NL);
     if (s == MUFFIN_OK) s = scan_input(P, P->stage_b, P->Lt, "delta");
     if (s != MUFFIN_OK) return s;
-    s = adjoint_fp64(P, P->stage_b, P->hhat, P->Lt, P->w64b, P->w64a);
+    s = adjoint(P, P->stage_b, 0, P->Lt, P->w64b, P->w64a, P->htd);
     if (s != MUFFIN_OK) return s;
-    CK(c64_real_to_f32(P->w64b, P->htd, scale, NL, P->ws));
     CK(axpy_f32(P->b, P->htd, (float)sp->eps, P->bbar, NL, P->ws));
     // per-band energies and weights
     std::vector<double> ysq(P->Lt);
@@ -1543,12 +1555,11 @@ muffin_status muffin_objective(muffin_plan P, const float *dirty, const float *x
   // +inf outside the positive orthant (the indicator of Eq. probopt)
   std::vector<int> neg(P->B, 0);
   if (P->p.positivity) {
-    std::vector<float> h(P->NL);
-    CK(cudaMemcpyAsync(h.data(), P->stage_b, P->NL * sizeof(float), cudaMemcpyDeviceToHost, P->ws));
-    CK(cudaStreamSynchronize(P->ws));
-    for (int c = 0; c < P->B; ++c)
-      for (size_t i = (size_t)c * P->NLc; i < (size_t)(c + 1) * P->NLc && !neg[c]; ++i)
-        if (h[i] < 0.f) neg[c] = 1;
+    std::vector<ImageStat> h;
+    s = image_scan(P, P->stage_b, P->Lt, h);
+    if (s != MUFFIN_OK) return s;
+    for (int l = 0; l < P->Lt; ++l)
+      if (h[l].negative) neg[l / P->L] = 1;
   }
   s = pi::leave(P, true);
   if (s != MUFFIN_OK) return s;
@@ -1711,9 +1722,11 @@ muffin_status muffin_op_gradient(muffin_plan P, const float *x, const float *dir
   const float *bb = nullptr;
   if (dirty) {
     s = fetch(P, dirty, P->stage_a, P->NL);
-    if (s == MUFFIN_OK) s = adjoint_fp64(P, P->stage_a, P->hhat, P->Lt, P->w64a, P->w64b);
+    if (s == MUFFIN_OK) {
+      CK(image_stats(P->stage_a, P->Lt, P->N, P->stat, P->ws));
+      s = adjoint(P, P->stage_a, 0, P->Lt, P->w64a, P->w64b, P->op_b);
+    }
     if (s != MUFFIN_OK) return s;
-    CK(c64_real_to_f32(P->w64a, P->op_b, 1.0 / ((double)P->n * P->n), P->NL, P->ws));
     bb = P->op_b;
   }
   s = fetch(P, x, P->op_in, P->NL);

@@ -64,6 +64,9 @@ struct muffin_plan_s {
   int *rec_count = nullptr;           // device counter of trace records
   double *dred = nullptr;             // reduction scratch
   double *wband = nullptr;            // [Lt]
+  muffin::ImageStat *stat = nullptr;  // [Lt] of the array scanned last
+  double *hmax = nullptr;             // [Lt] largest |h_hat|^2 of a band
+  float4 *twdd = nullptr;             // [n] twiddles as pairs of FP32 values
   double *records = nullptr;          // [max_records][B][7]
   int max_records = 0;
   float2 *S = nullptr;
@@ -168,7 +171,7 @@ muffin_status create(const muffin_params *p, const float *psf, const float *alph
                      const float *beta, void *stream, muffin_plan *out);
 // PSF spectra, |h_hat|^2 / n^2 and beta of cubes [b0, b1); psf holds b1-b0 cubes
 muffin_status load_psf(muffin_plan P, int b0, int b1, const float *psf);
-// b = H^T y for cubes [b0, b1) (FP64); dirty holds b1-b0 cubes
+// b = H^T y for cubes [b0, b1); dirty holds b1-b0 cubes
 muffin_status load_dirty(muffin_plan P, int b0, int b1, const float *dirty);
 // group g: cubes [b0, b1) restart from X0 (device, b1-b0 cubes; NULL = 0), U = V = T = 0
 muffin_status reset_cubes(muffin_plan P, int g, int b0, int b1, const float *x0_dev);

@@ -1,4 +1,4 @@
-// FP64 reductions: Lipschitz constant, per-band energies and the ADA-PT
+// FP64 reductions: per-band energies and the ADA-PT
 // statistics (Eqs. SUGAR, PSURE0) with the theta update of Eq. (adaptgrad).
 //
 // All reductions are deterministic: each block writes its partial sums and
@@ -13,16 +13,10 @@ namespace muffin {
 namespace {
 
 constexpr int kRedThreads = 256;
-constexpr int kMaxBlocks = 1024;
 
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __forceinline__ double warp_max(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
 
@@ -45,40 +39,6 @@ __device__ void block_sum(double (&v)[NV], double *sh /* [32][NV] */) {
     }
   }
   __syncthreads();
-}
-
-__global__ void k_max_abs2(const double2 *__restrict__ h, size_t count,
-                           double *__restrict__ part) {
-  double m = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const double2 z = h[i];
-    m = fmax(m, z.x * z.x + z.y * z.y);
-  }
-  __shared__ double sh[32];
-  m = warp_max(m);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    m = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-    m = warp_max(m);
-    if (threadIdx.x == 0) part[blockIdx.x] = m;
-  }
-}
-
-__global__ void k_max_final(const double *__restrict__ part, int nb,
-                            double *__restrict__ out) {
-  double m = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) m = fmax(m, part[i]);
-  __shared__ double sh[32];
-  m = warp_max(m);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    m = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-    m = warp_max(m);
-    if (threadIdx.x == 0) *out = m;
-  }
 }
 
 // grid (blocks_per_band, L); partials [L][blocks_per_band]
@@ -221,15 +181,6 @@ __global__ void k_theta_update(ThetaUpdateArgs a) {
 __global__ void k_bump(int *counter) { *counter += 1; }
 
 }  // namespace
-
-cudaError_t max_abs2_c64(const double2 *hh, size_t count, double *scratch,
-                         double *out, cudaStream_t st) {
-  size_t g = (count + kRedThreads - 1) / kRedThreads;
-  const int nb = (int)(g > kMaxBlocks ? kMaxBlocks : (g ? g : 1));
-  k_max_abs2<<<nb, kRedThreads, 0, st>>>(hh, count, scratch);
-  k_max_final<<<1, kRedThreads, 0, st>>>(scratch, nb, out);
-  return cudaGetLastError();
-}
 
 cudaError_t band_sumsq(const float *y, int L, size_t per_band, double *out,
                        cudaStream_t st) {

@@ -15,7 +15,7 @@ namespace muffin {
 
 namespace {
 
-// h_hat = (sqrt(m~), 0); chk = m with NaN where m < 0 (for the input scan)
+// h_hat [kx][ky] = (sqrt(m~), 0); chk = m with NaN where m < 0 (for the input scan)
 __global__ void k_vis_weights(const float *__restrict__ m, double2 *__restrict__ hh,
                               float *__restrict__ chk, int n, size_t nimg) {
   const size_t N = (size_t)n * n, total = N * nimg;
@@ -26,7 +26,7 @@ __global__ void k_vis_weights(const float *__restrict__ m, double2 *__restrict__
     const size_t mi = img * N + (size_t)((n - ky) & (n - 1)) * n + ((n - kx) & (n - 1));
     const float a = m[i], b = m[mi];
     const double ms = 0.5 * ((double)a + (double)b);
-    hh[i] = make_double2(ms > 0.0 ? sqrt(ms) : 0.0, 0.0);
+    hh[img * N + (size_t)kx * n + ky] = make_double2(ms > 0.0 ? sqrt(ms) : 0.0, 0.0);
     chk[i] = a >= 0.f ? a : __int_as_float(0x7fc00000);
   }
 }
