@@ -10,14 +10,25 @@
 //     P_0 + S_0[(P_1 - P_0) + S_1[(P_2 - P_1) + ... + S_{J-1}(P_J - P_{J-1})]]
 //     then m = x - tau (grad + mu_l s + t), x~ = (m)_+ (eqs. stpm, stpx).
 //
-// S_j is the separable B3 spline [1 4 6 4 1]/16 dilated by 2^j with periodic
-// boundaries.  One launch per scale, specialised on the dilation: a CTA
-// loads its 32 x 64 tile of every chain with a 2 * 2^j halo (wrapped) into
-// shared memory (four items per thread in flight), smooths it along y then
-// x, and does the scale's dual update (analysis) or Horner step
-// (synthesis); the running image of the next scale goes to a ping-pong
-// scratch.  The derivative chains use the primal's masks from the same
-// thread (Pi(p) per coefficient, U(m) per pixel).  J <= 4 (halo <= 16).
+// S_j is the separable B3 spline [1 4 6 4 1]/16 dilated by D = 2^j with periodic
+// boundaries.  One launch per scale and set of chains, specialised on D: a lane
+// owns one column of a 32 x 128 tile and its 2 D halo rows in registers (loaded
+// coalesced along the rows), smooths it along y there and puts the smoothed rows
+// into shared memory; after one barrier it smooths along x (five conflict-free
+// reads a pixel) and does the scale's dual update (analysis) or Horner step
+// (synthesis) on its own column, whose unsmoothed values it still holds.  U is
+// requested eight rows ahead.  The running image of the next scale goes to a
+// ping-pong scratch.  J <= 4 (halo <= 16).
+//
+// What bounds it: DRAM and the latency of a CTA's loads.  A tile with halo of all
+// chains in shared memory (two passes over it, 2 CTAs an SM) ran at 0.24-0.36 of
+// the copy bandwidth.  512 x 512 x 32, three chains, before and now: analysis 318
+// -> 122 us (first two scales, mean; 4.1 TB/s) and 195 -> 95, synthesis 328 and 201
+// -> 104 and 83 (4.8 TB/s), prox 257 -> 247 (its four arrays a row; requested two
+// rows ahead, and into L2 by the whole CTA first: 295 without).
+//
+// One chain a CTA: the primal's launch leaves its masks (Pi(p) per coefficient,
+// U(m) per pixel: a word of 32 rows a lane and plane) for the derivatives'.
 #include <cuda_runtime.h>
 
 #include <stdint.h>
@@ -28,23 +39,14 @@ namespace muffin {
 
 namespace {
 
-constexpr int IY = 32, IX = 64, INT = 256;   // output tile, threads
-constexpr int IQ = IY * IX / INT;              // outputs per thread (one column)
+constexpr int IY = 32, IX = 128, INT = 160;   // output tile, threads (a column each)
+constexpr int VP = INT;                       // floats of a smoothed row
+constexpr int RB = 8;                         // rows whose U is in flight
+static_assert(IX + 4 * 8 <= INT, "a column of the tile and its widest halo a thread");
 
 // B3 spline tap m of [1 4 6 4 1] / 16
 __device__ __forceinline__ constexpr float b3(int m) {
   return (m == 2 ? 6.f : (m == 1 || m == 3) ? 4.f : 1.f) * (1.f / 16.f);
-}
-
-// shared-memory geometry of a dilation D: input tile [IY + 4D][PA], vertical
-// pass [IY][PA] (odd pitch), per chain
-template <int D> struct Geo {
-  static constexpr int AY = IY + 4 * D, AX = IX + 4 * D;
-  static constexpr int PITCH = (AX & 1) ? AX : AX + 1;
-};
-template <int D>
-constexpr size_t iuwt_smem(int ch) {
-  return (size_t)ch * (Geo<D>::AY + IY) * Geo<D>::PITCH * sizeof(float);
 }
 
 struct IuwtArgs {
@@ -59,276 +61,315 @@ struct IuwtArgs {
   float *buf[2];                 // ping-pong running images [C][L][n][n]
   const float *beta;
   const DevScalars *sc;
+  uint32_t *masks;               // [L][tiles][min(n, IX)][2]
 };
 
-__device__ __forceinline__ int wrap(int v, int n) { return v & (n - 1); }
-
-// tile value of chain c at pixel pix for the source of analysis scale j
-template <int CH, int MODE>
-__device__ __forceinline__ void ana_src(const IuwtArgs &a, int l, size_t pix, float mu,
-                                        float (&w)[CH]) {
-  const size_t NN = (size_t)a.n * a.n, CS = (size_t)a.L * NN;
-  if (a.j == 0) {
-    if (MODE == WAVE_TRANSFORM) {
-      w[0] = a.in[(size_t)l * NN + pix];
-    } else {
-      float z[CH];
-#pragma unroll
-      for (int c = 0; c < CH; ++c) {
-        const size_t i = c * CS + (size_t)l * NN + pix;
-        z[c] = 2.f * a.xt[i] - a.x[i];
-      }
-      w[0] = z[0];
-      if (CH == 3) { w[1] = fmaf(mu, z[1], z[0]); w[2] = z[2]; }
-    }
-  } else {
-    const float *src = a.buf[a.j & 1];
-#pragma unroll
-    for (int c = 0; c < CH; ++c) w[c] = src[c * CS + (size_t)l * NN + pix];
-  }
-}
-
-// synthesis source of scale j: P_J - P_{J-1} at the coarsest step, else the
-// running image of scale j + 1
-template <int CH, int MODE>
-__device__ __forceinline__ void syn_src(const IuwtArgs &a, int l, size_t pix, float (&w)[CH]) {
-  const size_t NN = (size_t)a.n * a.n, CS = (size_t)a.L * NN;
-#pragma unroll
-  for (int c = 0; c < CH; ++c) {
-    if (a.j == a.J - 1) {
-      const float *u = (MODE == WAVE_TRANSFORM ? a.in : a.ur) +
-                       ((size_t)(c * a.L + l) * a.P) * NN + pix;
-      w[c] = u[(size_t)a.J * NN] - u[(size_t)(a.J - 1) * NN];
-    } else {
-      w[c] = a.buf[(a.j + 1) & 1][c * CS + (size_t)l * NN + pix];
-    }
-  }
-}
-
-// fill the wrapped input tile of every chain; LB items per thread per round
-// so their loads are in flight together
-template <int CH, int D, bool ANA, int MODE>
-__device__ __forceinline__ void load_tile(const IuwtArgs &a, float *A, int y0, int x0, int l,
-                                          float mu) {
-  using G = Geo<D>;
-  constexpr int LB = 4;
-  const int n = a.n;
-  constexpr int items = G::AY * G::AX;
-  for (int base = threadIdx.x; base < items; base += LB * INT) {
-    float w[LB][CH];
-#pragma unroll
-    for (int q = 0; q < LB; ++q) {
-      const int it = base + q * INT;
-      if (it < items) {
-        const int r = it / G::AX, col = it - r * G::AX;
-        const size_t pix = (size_t)wrap(y0 - 2 * D + r, n) * n + wrap(x0 - 2 * D + col, n);
-        if (ANA) ana_src<CH, MODE>(a, l, pix, mu, w[q]);
-        else syn_src<CH, MODE>(a, l, pix, w[q]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < LB; ++q) {
-      const int it = base + q * INT;
-      if (it < items) {
-        const int r = it / G::AX, col = it - r * G::AX;
-#pragma unroll
-        for (int c = 0; c < CH; ++c) A[(c * G::AY + r) * G::PITCH + col] = w[q][c];
-      }
-    }
-  }
-}
-
-// separable B3 smoothing at dilation D of chain c's resident tile -> out[q]
-// at the thread's pixels (rows ry + q * INT / IX of column rx)
+// y smoothing of the lane's column into shared memory, then (after the barrier)
+// x smoothing of row r at the lane's own pixel
 template <int D>
-__device__ __forceinline__ void smooth_tile(const float *A, float *Bv, int c, int ry, int rx,
-                                            float (&out)[IQ]) {
-  using G = Geo<D>;
-  const float *Ac = A + c * G::AY * G::PITCH;
-  float *Bc = Bv + c * IY * G::PITCH;
-  for (int it = threadIdx.x; it < IY * G::AX; it += INT) {
-    const int r = it / G::AX, col = it - r * G::AX;
+__device__ __forceinline__ void smooth_y(const float (&c)[IY + 4 * D], float *v) {
+#pragma unroll
+  for (int r = 0; r < IY; ++r) {
     float s = 0.f;
 #pragma unroll
-    for (int m = 0; m < 5; ++m) s = fmaf(b3(m), Ac[(r + m * D) * G::PITCH + col], s);
-    Bc[r * G::PITCH + col] = s;
+    for (int m = 0; m < 5; ++m) s = fmaf(b3(m), c[r + m * D], s);
+    v[r * VP] = s;
   }
-  __syncthreads();
+}
+template <int D>
+__device__ __forceinline__ float smooth_x(const float *v, int r) {
+  float s = 0.f;
 #pragma unroll
-  for (int q = 0; q < IQ; ++q) {
-    const int r = ry + q * (INT / IX);
-    float s = 0.f;
-#pragma unroll
-    for (int m = 0; m < 5; ++m) s = fmaf(b3(m), Bc[r * G::PITCH + rx + m * D], s);
-    out[q] = s;
+  for (int m = 0; m < 5; ++m) s = fmaf(b3(m), v[r * VP + (m - 2) * D], s);
+  return s;
+}
+
+struct Place {
+  unsigned xx, y0;               // the lane's column (wrapped) and the tile's first row
+  int lane;                      // column of the tile (halo: < 0 or >= IX)
+  bool own;                      // a pixel column of the image
+};
+template <int D>
+__device__ __forceinline__ Place place(int n) {
+  Place q;
+  const int ntx = (n + IX - 1) / IX;
+  const int x0 = (blockIdx.x % ntx) * IX;
+  q.y0 = (blockIdx.x / ntx) * IY;
+  q.lane = (int)threadIdx.x - 2 * D;
+  q.xx = (unsigned)(x0 + q.lane) & (n - 1);
+  q.own = q.lane >= 0 && q.lane < IX && x0 + q.lane < n;
+  return q;
+}
+
+// the tile's rows of an image into L2: a 128-byte line a thread and round
+__device__ __forceinline__ void prefetch_tile(const float *img, unsigned n, unsigned y0) {
+  const int ntx = (n + IX - 1) / IX;
+  const unsigned x0 = (blockIdx.x % ntx) * IX;
+  for (unsigned i = threadIdx.x; i < IY * (IX / 32); i += INT) {
+    const unsigned x = x0 + 32 * (i % (IX / 32)), y = y0 + i / (IX / 32);
+    if (x < n && y < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(img + (size_t)y * n + x));
   }
 }
 
-template <int CH, int MODE, int D>
-__global__ void __launch_bounds__(INT) k_iuwt_ana(IuwtArgs a) {
-  using G = Geo<D>;
-  extern __shared__ float ism[];
-  float *A = ism;                        // [CH][AY][PITCH]
-  float *Bv = A + CH * G::AY * G::PITCH; // [CH][IY][PITCH]
-  const int n = a.n;
-  const int ntx = (n + IX - 1) / IX;
-  const int x0 = (blockIdx.x % ntx) * IX, y0 = (blockIdx.x / ntx) * IY;
-  const int l = blockIdx.y;
+// chain c = 0 (DERIV = false; masks recorded where a.masks is set), or
+// 1 + blockIdx.z
+template <int MODE, int D, bool LAST, bool DERIV>
+__global__ void __launch_bounds__(INT, 3) k_iuwt_ana(IuwtArgs a) {
+  __shared__ float vs[IY * VP];
+  const unsigned n = a.n, nm = n - 1;
+  const int l = blockIdx.y, c = DERIV ? 1 + blockIdx.z : 0, tid = threadIdx.x;
+  const Place w = place<D>(n);
   const size_t NN = (size_t)n * n, CS = (size_t)a.L * NN;
-  float mu = 0.f, sbl = 1.f;
+  float mu = 0.f, q = 1.f;
   if (MODE == WAVE_ITERATE) {
     const DevScalars &S = a.sc[l / a.Lc];
     mu = (float)S.mu;
-    sbl = (float)(S.sigma * (double)a.beta[l]);
+    q = (float)(S.sigma * (double)a.beta[l]);
+    if (c != 1) q *= mu;
   }
-  load_tile<CH, D, true, MODE>(a, A, y0, x0, l, mu);
+  float col[IY + 4 * D];
+  if (tid < IX + 4 * D) {
+    const size_t i0 = c * CS + l * NN + w.xx;
+    const float *src = D == 1 ? nullptr : a.buf[a.j & 1] + i0;
+    const float *xt = a.xt + i0, *x = (MODE == WAVE_TRANSFORM && D == 1 ? a.in : a.x) + i0;
+#pragma unroll
+    for (int i = 0; i < IY + 4 * D; ++i) {
+      const unsigned o = ((w.y0 + i - 2 * D) & nm) * n;
+      if (D > 1) col[i] = src[o];
+      else col[i] = MODE == WAVE_TRANSFORM ? x[o] : 2.f * xt[o] - x[o];
+    }
+    if (D == 1 && DERIV && c == 1) {                 // Algorithm 3 input: z0 + mu z1
+      xt -= CS;
+      x -= CS;
+#pragma unroll
+      for (int i = 0; i < IY + 4 * D; ++i) {
+        const unsigned o = ((w.y0 + i - 2 * D) & nm) * n;
+        col[i] = fmaf(mu, col[i], 2.f * xt[o] - x[o]);
+      }
+    }
+    smooth_y<D>(col, vs + tid);
+  }
+  constexpr int NP = LAST ? 2 : 1;
+  float *uj = a.u + ((size_t)(c * a.L + l) * a.P + a.j) * NN + (size_t)w.y0 * n + w.xx;
+  float u[2][NP][RB];
+  auto request = [&](int r0, float (&d)[NP][RB]) {   // planes j (and J = j + 1) of 8 rows
+    if (MODE == WAVE_ITERATE && w.own)
+#pragma unroll
+      for (int p = 0; p < NP; ++p)
+#pragma unroll
+        for (int r = 0; r < RB; ++r)
+          d[p][r] = w.y0 + r0 + r < n ? uj[p * NN + (size_t)(r0 + r) * n] : 0.f;
+  };
+  request(0, u[0]);
+  uint32_t *mk = a.masks && w.own
+                     ? a.masks + (((size_t)l * gridDim.x + blockIdx.x) * (n < IX ? n : IX) + w.lane) * 2
+                     : nullptr;
+  uint32_t keep[2] = {0u, 0u};
+  if (DERIV && w.own) {
+    keep[0] = mk[0];
+    if (LAST) keep[1] = mk[1];
+  }
   __syncthreads();
-  const int rx = threadIdx.x % IX, ry = threadIdx.x / IX;
-  const bool last = a.j == a.J - 1;
-  uint32_t keep = 0;
-#pragma unroll 1
-  for (int c = 0; c < CH; ++c) {
-    float cn[IQ];
-    smooth_tile<D>(A, Bv, c, ry, rx, cn);
-    const float q = MODE == WAVE_ITERATE ? (c == 1 ? sbl : sbl * mu) : 1.f;
+  if (!w.own) return;
+  float *nxt = LAST ? nullptr : a.buf[(a.j + 1) & 1] + c * CS + l * NN + (size_t)w.y0 * n + w.xx;
 #pragma unroll
-    for (int k = 0; k < IQ; ++k) {
-      const int r = ry + k * (INT / IX);
-      const int yy = y0 + r, xx = x0 + rx;
-      if (yy >= n || xx >= n) continue;
-      const float cj = A[(c * G::AY + r + 2 * D) * G::PITCH + rx + 2 * D];
-      const size_t pix = (size_t)yy * n + xx;
-      float *up = a.u + ((size_t)(c * a.L + l) * a.P) * NN + pix;
-      // planes j (detail) and, at the last scale, J (coarse)
+  for (int r0 = 0; r0 < IY; r0 += RB) {
+    const int cur = (r0 / RB) & 1;
+    if (r0 + RB < IY) request(r0 + RB, u[cur ^ 1]);
 #pragma unroll
-      for (int s = 0; s < 2; ++s) {
-        if (s == 1 && !last) break;
-        const float val = s == 0 ? cj - cn[k] : cn[k];
-        float *uq = up + (size_t)(s == 0 ? a.j : a.J) * NN;
-        if (MODE == WAVE_TRANSFORM) {
-          *uq = val;
-        } else {
-          const float p = fmaf(q, val, *uq);
-          const uint32_t bit = 1u << (2 * k + s);
-          if (c == 0) {
-            *uq = satf(p);
-            if (fabsf(p) <= 1.0f) keep |= bit;
+    for (int k = 0; k < RB; ++k) {
+      const int r = r0 + k;
+      const float cn = smooth_x<D>(vs + tid, r);
+      if (w.y0 + r >= n) continue;
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        float val = p == 0 ? col[r + 2 * D] - cn : cn;
+        if (MODE == WAVE_ITERATE) {
+          const float t = fmaf(q, val, u[cur][p][k]);
+          if (DERIV) {
+            val = (keep[p] >> r) & 1u ? t : 0.f;
           } else {
-            *uq = (keep & bit) ? p : 0.f;
+            val = satf(t);
+            if (fabsf(t) <= 1.0f) keep[p] |= 1u << r;
           }
         }
+        uj[p * NN + (size_t)r * n] = val;
       }
-      if (!last) a.buf[(a.j + 1) & 1][c * CS + (size_t)l * NN + pix] = cn[k];
+      if (!LAST) nxt[(size_t)r * n] = cn;
     }
+  }
+  if (MODE == WAVE_ITERATE && !DERIV && mk) {
+    mk[0] = keep[0];
+    if (LAST) mk[1] = keep[1];
   }
 }
 
-template <int CH, int MODE, int D>
-__global__ void __launch_bounds__(INT) k_iuwt_syn(IuwtArgs a) {
-  using G = Geo<D>;
-  extern __shared__ float ism[];
-  float *A = ism;
-  float *Bv = A + CH * G::AY * G::PITCH;
-  const int n = a.n;
-  const int ntx = (n + IX - 1) / IX;
-  const int x0 = (blockIdx.x % ntx) * IX, y0 = (blockIdx.x / ntx) * IY;
-  const int l = blockIdx.y;
-  const size_t NN = (size_t)n * n, CS = (size_t)a.L * NN;
-  load_tile<CH, D, false, MODE>(a, A, y0, x0, l, 0.f);
-  __syncthreads();
-  const int rx = threadIdx.x % IX, ry = threadIdx.x / IX;
-  float o[CH][IQ];
-#pragma unroll 1
-  for (int c = 0; c < CH; ++c) {
-    float sr[IQ];
-    smooth_tile<D>(A, Bv, c, ry, rx, sr);
+// TOP: the coarsest step (source P_J - P_{J-1}); otherwise the running image of
+// scale j + 1.  Scales j > 0 take chains blockIdx.z; j = 0 (D = 1) ends in the
+// prox, chain 0 or chains 1 + blockIdx.z.
+template <int MODE, int D, bool TOP, bool DERIV>
+__global__ void __launch_bounds__(INT, 3) k_iuwt_syn(IuwtArgs a) {
+  __shared__ float vs[IY * VP];
+  const unsigned n = a.n, nm = n - 1;
+  const int l = blockIdx.y, c = (DERIV ? 1 : 0) + blockIdx.z, tid = threadIdx.x;
+  const Place w = place<D>(n);
+  const size_t NN = (size_t)n * n, CS = (size_t)a.L * NN, US = CS * a.P;
+  // chain 1's W^T u + mu W^T u'_mu (Algorithm 3) by linearity, from mixed inputs
+  const bool mix = D == 1 && DERIV && c == 1;
+  const float mu = MODE == WAVE_ITERATE && D == 1 ? (float)a.sc[l / a.Lc].mu : 0.f;
+  const float *ub = (MODE == WAVE_TRANSFORM ? a.in : a.ur) + c * US + (size_t)l * a.P * NN;
+  if (D == 1 && MODE == WAVE_ITERATE) {
+    const size_t o = c * CS + l * NN;
+    prefetch_tile(ub, n, w.y0);
+    prefetch_tile(a.x + o, n, w.y0);
+    prefetch_tile(a.g + o, n, w.y0);
+    prefetch_tile(a.t + o, n, w.y0);
+  }
+  float col[IY + 4 * D];
+  if (tid < IX + 4 * D) {
+    const float *s1 = TOP ? ub + (size_t)a.J * NN + w.xx
+                          : a.buf[(a.j + 1) & 1] + c * CS + l * NN + w.xx;
+    const float *s2 = ub + (size_t)(a.J - 1) * NN + w.xx;
 #pragma unroll
-    for (int k = 0; k < IQ; ++k) {
-      const int yy = y0 + ry + k * (INT / IX), xx = x0 + rx;
-      o[c][k] = 0.f;
-      if (yy >= n || xx >= n) continue;
-      const size_t pix = (size_t)yy * n + xx;
-      const float *u = (MODE == WAVE_TRANSFORM ? a.in : a.ur) +
-                       ((size_t)(c * a.L + l) * a.P) * NN + pix;
-      if (a.j > 0) {
-        const float v = sr[k] + u[(size_t)a.j * NN] - u[(size_t)(a.j - 1) * NN];
-        a.buf[a.j & 1][c * CS + (size_t)l * NN + pix] = v;
-      } else {
-        o[c][k] = u[0] + sr[k];
+    for (int i = 0; i < IY + 4 * D; ++i) {
+      const unsigned o = ((w.y0 + i - 2 * D) & nm) * n;
+      col[i] = TOP ? s1[o] - s2[o] : s1[o];
+    }
+    if (mix) {
+      s1 -= TOP ? US : CS;
+      s2 -= US;
+#pragma unroll
+      for (int i = 0; i < IY + 4 * D; ++i) {
+        const unsigned o = ((w.y0 + i - 2 * D) & nm) * n;
+        col[i] = fmaf(mu, col[i], TOP ? s1[o] - s2[o] : s1[o]);
       }
     }
+    smooth_y<D>(col, vs + tid);
   }
-  if (a.j > 0) return;
-  const float mu = (MODE == WAVE_ITERATE) ? (float)a.sc[l / a.Lc].mu : 0.f;
-  const float tau = (MODE == WAVE_ITERATE) ? (float)a.sc[l / a.Lc].tau : 0.f;
-  const float bl = (MODE == WAVE_ITERATE) ? a.beta[l] : 0.f;
+  __syncthreads();
+  if (!w.own) return;
+  const size_t i0 = (size_t)w.y0 * n + w.xx;
+  if constexpr (D > 1) {
+    const float *uj = ub + (size_t)a.j * NN + i0;
+    float *dst = a.buf[a.j & 1] + c * CS + l * NN + i0;
+    float d[2][RB];
+    auto request = [&](int r0, float (&v)[RB]) {
 #pragma unroll
-  for (int k = 0; k < IQ; ++k) {
-    const int yy = y0 + ry + k * (INT / IX), xx = x0 + rx;
-    if (yy >= n || xx >= n) continue;
-    const size_t i0 = (size_t)l * NN + (size_t)yy * n + xx;
-    if (MODE == WAVE_TRANSFORM) {
-      a.out[i0] = o[0][k];
-      continue;
-    }
-    // W^T of chain 1 by linearity: W^T u + mu W^T u'_mu (Algorithm 3)
-    float acc[CH];
-    acc[0] = o[0][k];
-    if (CH == 3) { acc[1] = fmaf(mu, o[1][k], o[0][k]); acc[2] = o[2][k]; }
-    bool keep = true;
+      for (int r = 0; r < RB; ++r) {
+        const size_t o = (size_t)(r0 + r) * n;
+        v[r] = 0.f;
+        if (w.y0 + r0 + r < n) v[r] = uj[o] - (uj - NN)[o];
+      }
+    };
+    request(0, d[0]);
 #pragma unroll
-    for (int c = 0; c < CH; ++c) {
-      const float sc = (CH == 3 && c == 1) ? bl : bl * mu;   // mu_l, beta_l, mu_l
-      const size_t i = c * CS + i0;
-      const float m = a.x[i] - tau * (a.g[i] + sc * acc[c] + a.t[i]);
-      if (c == 0) keep = !a.positivity || m > 0.f;
-      a.xt_out[i] = keep ? m : 0.f;
+    for (int r0 = 0; r0 < IY; r0 += RB) {
+      const int cur = (r0 / RB) & 1;
+      if (r0 + RB < IY) request(r0 + RB, d[cur ^ 1]);
+#pragma unroll
+      for (int k = 0; k < RB; ++k) {
+        const float s = smooth_x<D>(vs + tid, r0 + k);
+        if (w.y0 + r0 + k < n) dst[(size_t)(r0 + k) * n] = s + d[cur][k];
+      }
     }
+  } else {
+    uint32_t *mk = a.masks ? a.masks + (((size_t)l * gridDim.x + blockIdx.x) * (n < IX ? n : IX) + w.lane) * 2
+                           : nullptr;
+    uint32_t keep = DERIV ? mk[0] : 0u;
+    const float tau = MODE == WAVE_ITERATE ? (float)a.sc[l / a.Lc].tau : 0.f;
+    const float bl = MODE == WAVE_ITERATE ? a.beta[l] : 0.f;
+    const float sc = c == 1 ? bl : bl * mu;          // mu_l, beta_l, mu_l
+    const size_t i1 = c * CS + l * NN + i0;
+    constexpr int RQ = 2;                            // four arrays a row: 2 x 2 rows in flight
+    float in[2][4][RQ];
+    auto request = [&](int r0, float (&v)[4][RQ]) {
+#pragma unroll
+      for (int r = 0; r < RQ; ++r) {
+        if (w.y0 + r0 + r >= n) continue;
+        const size_t o = (size_t)(r0 + r) * n;
+        v[0][r] = ub[i0 + o];
+        if (mix) v[0][r] = fmaf(mu, v[0][r], (ub - US)[i0 + o]);
+        if (MODE == WAVE_ITERATE) {
+          v[1][r] = a.x[i1 + o];
+          v[2][r] = a.g[i1 + o];
+          v[3][r] = a.t[i1 + o];
+        }
+      }
+    };
+    request(0, in[0]);
+#pragma unroll
+    for (int r0 = 0; r0 < IY; r0 += RQ) {
+      const int cur = (r0 / RQ) & 1;
+      if (r0 + RQ < IY) request(r0 + RQ, in[cur ^ 1]);
+#pragma unroll
+      for (int k = 0; k < RQ; ++k) {
+        const int r = r0 + k;
+        const float s = smooth_x<D>(vs + tid, r);
+        if (w.y0 + r >= n) continue;
+        const float acc = in[cur][0][k] + s;
+        const size_t o = i1 + (size_t)r * n;
+        if (MODE == WAVE_TRANSFORM) {
+          a.out[o] = acc;
+          continue;
+        }
+        const float m = in[cur][1][k] - tau * (in[cur][2][k] + sc * acc + in[cur][3][k]);
+        bool ok;
+        if (DERIV) {
+          ok = (keep >> r) & 1u;
+        } else {
+          ok = !a.positivity || m > 0.f;
+          if (ok) keep |= 1u << r;
+        }
+        a.xt_out[o] = ok ? m : 0.f;
+      }
+    }
+    if (MODE == WAVE_ITERATE && !DERIV && mk) mk[0] = keep;
   }
 }
 
 inline int itiles(int n) { return ((n + IX - 1) / IX) * ((n + IY - 1) / IY); }
 
 template <int CH, int MODE, int D>
-cudaError_t launch_ana_d(const IuwtArgs &a, int L, int n, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_iuwt_ana<CH, MODE, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)iuwt_smem<D>(CH));
-    attr = true;
+void launch_ana_d(const IuwtArgs &a, cudaStream_t st) {
+  const dim3 g(itiles(a.n), a.L), g2(itiles(a.n), a.L, 2);
+  if (a.j == a.J - 1) {
+    k_iuwt_ana<MODE, D, true, false><<<g, INT, 0, st>>>(a);
+    if constexpr (CH == 3) k_iuwt_ana<MODE, D, true, true><<<g2, INT, 0, st>>>(a);
+  } else {
+    k_iuwt_ana<MODE, D, false, false><<<g, INT, 0, st>>>(a);
+    if constexpr (CH == 3) k_iuwt_ana<MODE, D, false, true><<<g2, INT, 0, st>>>(a);
   }
-  k_iuwt_ana<CH, MODE, D><<<dim3(itiles(n), L), INT, iuwt_smem<D>(CH), st>>>(a);
-  return cudaGetLastError();
 }
 
 template <int CH, int MODE, int D>
-cudaError_t launch_syn_d(const IuwtArgs &a, int L, int n, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_iuwt_syn<CH, MODE, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)iuwt_smem<D>(CH));
-    attr = true;
+void launch_syn_d(const IuwtArgs &a, cudaStream_t st) {
+  const bool top = a.j == a.J - 1;
+  const dim3 g(itiles(a.n), a.L, D > 1 ? CH : 1), g2(itiles(a.n), a.L, 2);
+  if (top) k_iuwt_syn<MODE, D, true, false><<<g, INT, 0, st>>>(a);
+  else k_iuwt_syn<MODE, D, false, false><<<g, INT, 0, st>>>(a);
+  if constexpr (CH == 3 && D == 1) {
+    if (top) k_iuwt_syn<MODE, D, true, true><<<g2, INT, 0, st>>>(a);
+    else k_iuwt_syn<MODE, D, false, true><<<g2, INT, 0, st>>>(a);
   }
-  k_iuwt_syn<CH, MODE, D><<<dim3(itiles(n), L), INT, iuwt_smem<D>(CH), st>>>(a);
-  return cudaGetLastError();
 }
 
 template <int CH, int MODE>
 cudaError_t ana_all(const WaveArgs &w, IuwtArgs a, cudaStream_t st) {
   const double vox = (double)CH * w.L * w.n * w.n;
+  if (CH == 1) a.masks = nullptr;
   for (int j = 0; j < w.J; ++j) {
     a.j = j;
     const double bytes = vox * ((j == 0 && MODE == WAVE_ITERATE ? 8.0 : 4.0) +
                                 (MODE == WAVE_ITERATE ? 8.0 : 4.0) * (j == w.J - 1 ? 2 : 1) +
                                 (j == w.J - 1 ? 0.0 : 4.0));
     ProfScope ps(w.prof, "iuwt_ana_dual", bytes, vox * 22.0, st);
-    cudaError_t e;
     switch (j) {
-      case 0: e = launch_ana_d<CH, MODE, 1>(a, w.L, w.n, st); break;
-      case 1: e = launch_ana_d<CH, MODE, 2>(a, w.L, w.n, st); break;
-      case 2: e = launch_ana_d<CH, MODE, 4>(a, w.L, w.n, st); break;
-      default: e = launch_ana_d<CH, MODE, 8>(a, w.L, w.n, st); break;
+      case 0: launch_ana_d<CH, MODE, 1>(a, st); break;
+      case 1: launch_ana_d<CH, MODE, 2>(a, st); break;
+      case 2: launch_ana_d<CH, MODE, 4>(a, st); break;
+      default: launch_ana_d<CH, MODE, 8>(a, st); break;
     }
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -337,18 +378,19 @@ cudaError_t ana_all(const WaveArgs &w, IuwtArgs a, cudaStream_t st) {
 template <int CH, int MODE>
 cudaError_t syn_all(const WaveArgs &w, IuwtArgs a, cudaStream_t st) {
   const double vox = (double)CH * w.L * w.n * w.n;
+  if (CH == 1) a.masks = nullptr;
   for (int j = w.J - 1; j >= 0; --j) {
     a.j = j;
     const double bytes = vox * ((j == w.J - 1 ? 8.0 : 4.0) + 8.0 * (j > 0) + 4.0 * (j == 0) +
                                 (j > 0 ? 4.0 : (MODE == WAVE_ITERATE ? 16.0 : 4.0)));
     ProfScope ps(w.prof, j == 0 ? "iuwt_syn_prox" : "iuwt_syn", bytes, vox * 22.0, st);
-    cudaError_t e;
     switch (j) {
-      case 0: e = launch_syn_d<CH, MODE, 1>(a, w.L, w.n, st); break;
-      case 1: e = launch_syn_d<CH, MODE, 2>(a, w.L, w.n, st); break;
-      case 2: e = launch_syn_d<CH, MODE, 4>(a, w.L, w.n, st); break;
-      default: e = launch_syn_d<CH, MODE, 8>(a, w.L, w.n, st); break;
+      case 0: launch_syn_d<CH, MODE, 1>(a, st); break;
+      case 1: launch_syn_d<CH, MODE, 2>(a, st); break;
+      case 2: launch_syn_d<CH, MODE, 4>(a, st); break;
+      default: launch_syn_d<CH, MODE, 8>(a, st); break;
     }
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -357,7 +399,7 @@ cudaError_t syn_all(const WaveArgs &w, IuwtArgs a, cudaStream_t st) {
 IuwtArgs base_args(const WaveArgs &w, int C) {
   IuwtArgs a{};
   a.n = w.n; a.L = w.L; a.Lc = w.Lc > 0 ? w.Lc : w.L; a.P = w.J + 1; a.J = w.J;
-  a.beta = w.beta; a.sc = w.sc;
+  a.beta = w.beta; a.sc = w.sc; a.masks = w.masks;
   const size_t cl = (size_t)C * w.L * w.n * w.n;
   a.buf[0] = w.scratch;
   a.buf[1] = w.scratch + cl;
