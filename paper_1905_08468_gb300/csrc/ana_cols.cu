@@ -147,11 +147,11 @@ __device__ __forceinline__ void store_item(float *p, const float (&w)[Q]) {
 // Chain 0 (DERIV = false; records the masks when a.masks is set) or the chains
 // 1 + blockIdx.z of the derivatives.  SRC_LL: one basis a CTA (blockIdx.y =
 // band * K + basis) of the previous level's approximations; otherwise level 1,
-// all bases.  CTAs an SM: as many as keep the column in registers unspilled
+// all bases, or (SPLIT) one of `groups` shares of them.  CTAs an SM: as many as keep the column in registers unspilled
 // (the derivatives' code needs more of them).
-template <int CY, int SRC, bool LAST, bool DERIV>
+template <int CY, int SRC, bool LAST, bool DERIV, bool SPLIT>
 __global__ void __launch_bounds__(NT, DERIV ? (CY == 16 ? 2 : 3) : (CY == 16 ? 3 : 4))
-k_ana_cols(AnaArgs a, bool iterate) {
+k_ana_cols(AnaArgs a, bool iterate, int groups) {
   using T = Tile<CY>;
   constexpr int Q = T::Q;
   extern __shared__ float vbuf[];                   // [2][low, high][CY][VP]
@@ -160,8 +160,10 @@ k_ana_cols(AnaArgs a, bool iterate) {
   const unsigned n = a.n, M = SRC == SRC_LL ? a.M : n, h = M >> 1, Mm = M - 1, hn = h * n;
   const unsigned ntx = (h + CX - 1) / CX;
   const unsigned kx0 = (blockIdx.x % ntx) * CX, ky0 = (blockIdx.x / ntx) * CY;
-  const int K = a.K, l = SRC == SRC_LL ? blockIdx.y / K : blockIdx.y;
-  const int b0 = SRC == SRC_LL ? blockIdx.y % K : 0, b1 = SRC == SRC_LL ? b0 + 1 : K;
+  // bases b0, b0 + step, ... below b1
+  const int K = a.K, shares = SRC == SRC_LL ? K : SPLIT ? groups : 1, l = blockIdx.y / shares;
+  const int step = SRC == SRC_LL ? 1 : shares;
+  const int b0 = blockIdx.y % shares, b1 = SRC == SRC_LL ? b0 + 1 : K;
   const int c = DERIV ? 1 + blockIdx.z : 0;
   const size_t NN = (size_t)n * n, CS = (size_t)a.L * NN;
   float mu = 0.f, q = 1.f;
@@ -225,7 +227,7 @@ k_ana_cols(AnaArgs a, bool iterate) {
                          : nullptr;
   int buf = 0;
 #pragma unroll 1
-  for (int b = b0; b < b1; ++b) {
+  for (int b = b0; b < b1; b += step) {
     const size_t img = (size_t)(c * a.L + l) * K + b;
     float *ub = a.u + img * NN;
     uint32_t keep = 0;
@@ -237,12 +239,12 @@ k_ana_cols(AnaArgs a, bool iterate) {
       if (LAST) load_item(u[LAST ? 3 : 0], ub + uo);
       if (DERIV) keep = mk[(size_t)b * gridDim.x * T::ITEMS];
     }
-    if (SRC == SRC_ITERATE && tid < 6 * CY && b + 1 < b1) {
+    if (SRC == SRC_ITERATE && tid < 6 * CY && b + step < b1) {
       // the next step's U tile into L2, a 128-byte line a thread
       const int sb = (tid % 6) >> 1;
       const unsigned px = kx0 + 32 * (tid & 1), py = ky0 + tid / 6;
       if (px < h && py < h) {
-        const float *p = ub + NN + (py * n + px) + (sb == 0 ? h : sb == 1 ? hn : hn + h);
+        const float *p = ub + step * NN + (py * n + px) + (sb == 0 ? h : sb == 1 ? hn : hn + h);
         asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
       }
     }
@@ -299,12 +301,26 @@ cudaError_t launch(const AnaArgs &a, int chains, bool iterate, cudaStream_t st) 
   constexpr size_t sm = (size_t)(SRC == SRC_LL ? 1 : 2) * T::VB * sizeof(float);
   static_assert(sm <= 48 * 1024, "no opt-in for more shared memory");
   const int h = a.M >> 1, nt = ((h + CX - 1) / CX) * ((h + CY - 1) / CY);
-  const int ny = SRC == SRC_LL ? a.L * a.K : a.L;
+  // level 1 with few tiles: the bases dealt to CTAs of their own while all fit
+  // one wave of the 8-row tiles (64 x 64 x 8: 14.2 -> 8.5 us)
+  int groups = 1;
+  if (CY == 8 && SRC != SRC_LL)
+    while (2 * groups <= a.K && (long long)nt * a.L * 2 * groups <= 608) groups *= 2;
+  const int ny = a.L * (SRC == SRC_LL ? a.K : groups);
   AnaArgs g = a;
   if (chains == 1) g.masks = nullptr;
-  k_ana_cols<CY, SRC, LAST, false><<<dim3(nt, ny), NT, sm, st>>>(g, iterate);
+  const dim3 g1(nt, ny), g2(nt, ny, 2);
+  if constexpr (CY == 8 && SRC != SRC_LL) {
+    if (groups > 1) {
+      k_ana_cols<CY, SRC, LAST, false, true><<<g1, NT, sm, st>>>(g, iterate, groups);
+      if constexpr (SRC != SRC_OPERATOR)
+        if (chains == 3) k_ana_cols<CY, SRC, LAST, true, true><<<g2, NT, sm, st>>>(g, iterate, groups);
+      return cudaGetLastError();
+    }
+  }
+  k_ana_cols<CY, SRC, LAST, false, false><<<g1, NT, sm, st>>>(g, iterate, 1);
   if constexpr (SRC != SRC_OPERATOR)
-    if (chains == 3) k_ana_cols<CY, SRC, LAST, true><<<dim3(nt, ny, 2), NT, sm, st>>>(g, iterate);
+    if (chains == 3) k_ana_cols<CY, SRC, LAST, true, false><<<g2, NT, sm, st>>>(g, iterate, 1);
   return cudaGetLastError();
 }
 
