@@ -31,6 +31,7 @@
 // chain 57.6 -> 33.7 us; three chains 1024 x 1024 x 64 2.91 -> 2.49 ms.
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "kernels.h"
 #include "wavelet.h"
 
@@ -152,6 +153,7 @@ __device__ __forceinline__ void store_item(float *p, const float (&w)[Q]) {
 template <int CY, int SRC, bool LAST, bool DERIV, bool SPLIT>
 __global__ void __launch_bounds__(NT, DERIV ? (CY == 16 ? 2 : 3) : (CY == 16 ? 3 : 4))
 k_ana_cols(AnaArgs a, bool iterate, int groups) {
+  chain_enter();
   using T = Tile<CY>;
   constexpr int Q = T::Q;
   extern __shared__ float vbuf[];                   // [2][low, high][CY][VP]
@@ -312,15 +314,15 @@ cudaError_t launch(const AnaArgs &a, int chains, bool iterate, cudaStream_t st) 
   const dim3 g1(nt, ny), g2(nt, ny, 2);
   if constexpr (CY == 8 && SRC != SRC_LL) {
     if (groups > 1) {
-      k_ana_cols<CY, SRC, LAST, false, true><<<g1, NT, sm, st>>>(g, iterate, groups);
+      launch_chain(k_ana_cols<CY, SRC, LAST, false, true>, g1, NT, sm, st, g, iterate, groups);
       if constexpr (SRC != SRC_OPERATOR)
-        if (chains == 3) k_ana_cols<CY, SRC, LAST, true, true><<<g2, NT, sm, st>>>(g, iterate, groups);
+        if (chains == 3) launch_chain(k_ana_cols<CY, SRC, LAST, true, true>, g2, NT, sm, st, g, iterate, groups);
       return cudaGetLastError();
     }
   }
-  k_ana_cols<CY, SRC, LAST, false, false><<<g1, NT, sm, st>>>(g, iterate, 1);
+  launch_chain(k_ana_cols<CY, SRC, LAST, false, false>, g1, NT, sm, st, g, iterate, 1);
   if constexpr (SRC != SRC_OPERATOR)
-    if (chains == 3) k_ana_cols<CY, SRC, LAST, true, false><<<g2, NT, sm, st>>>(g, iterate, 1);
+    if (chains == 3) launch_chain(k_ana_cols<CY, SRC, LAST, true, false>, g2, NT, sm, st, g, iterate, 1);
   return cudaGetLastError();
 }
 

@@ -31,6 +31,7 @@
 
 #include <algorithm>
 
+#include "chain.cuh"
 #include "kernels.h"
 
 namespace muffin {
@@ -89,6 +90,7 @@ __device__ __forceinline__ void half_product(const float *__restrict__ A, int Mp
 // RB: rows of a task of C^T v
 template <int CH, int MODE, int PT, int RB>
 __global__ void __launch_bounds__(DT, 3) k_dct_fold(FoldArgs a) {
+  chain_enter();
   constexpr int PG = PT / 4;                      // pixel groups
   const int NG = blockDim.x / PG;                 // row groups in flight
   extern __shared__ float sm[];
@@ -271,7 +273,7 @@ cudaError_t launch_fold_r(FoldArgs &a, int ctas_per_sm, size_t sm, cudaStream_t 
   ProfScope ps(prof, MODE == WAVE_ITERATE ? "spectral_dual" : "spectral_op",
                MODE == WAVE_ITERATE ? CH * vox * 20.0 : vox * 8.0,
                (MODE == WAVE_ITERATE ? 2.0 : 1.0) * CH * a.L * vox, st);
-  k_dct_fold<CH, MODE, PT, RB><<<grid, threads, sm, st>>>(a);
+  launch_chain(k_dct_fold<CH, MODE, PT, RB>, grid, threads, sm, st, a);
   return cudaGetLastError();
 }
 

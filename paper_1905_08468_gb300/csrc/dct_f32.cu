@@ -36,6 +36,7 @@
 #include <cmath>
 
 #include "fft32.cuh"
+#include "chain.cuh"
 #include "kernels.h"
 
 namespace muffin {
@@ -89,6 +90,7 @@ __device__ __forceinline__ int mpos(int l) {
 
 template <int L, int CH, int MODE, int FT>
 __global__ void __launch_bounds__(FT, FT == 64 ? 6 : 2) k_dct_f32(F32Args a) {
+  chain_enter();
   using S = FShape<L, FT>;
   constexpr int NB = S::NB, PT = S::PT, PITCH = S::PITCH;
   extern __shared__ float2 fsm[];
@@ -290,7 +292,7 @@ cudaError_t launch_f32_t(const F32Args &a, cudaStream_t st, Prof *prof) {
                (MODE == WAVE_ITERATE ? 2.0 : 1.0) * CH * vox * (2.5 * std::log2((double)L) + 6.0),
                st);
   const unsigned gx = (unsigned)((a.npix + S::PT - 1) / S::PT);
-  k_dct_f32<L, CH, MODE, FT><<<dim3(gx, a.B), FT, sm, st>>>(a);
+  launch_chain(k_dct_f32<L, CH, MODE, FT>, dim3(gx, a.B), FT, sm, st, a);
   return cudaGetLastError();
 }
 

@@ -29,6 +29,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "kernels.h"
 
 namespace muffin {
@@ -203,6 +204,7 @@ __device__ __forceinline__ void store_split(uint8_t *ahi, uint8_t *alo, int row,
 
 template <int CH>
 __global__ void __launch_bounds__(CTA_T, 1) k_dct_tc(TcArgs a) {
+  chain_enter();
   extern __shared__ uint8_t raw[];
   __shared__ __align__(8) uint64_t mbar[NG];
   __shared__ uint32_t tmem_base;
@@ -391,7 +393,7 @@ cudaError_t launch_tc(const TcArgs &a, cudaStream_t st, Prof *prof) {
   const size_t grid = ctas < (size_t)sms ? ctas : (size_t)sms;
   const double vox = (double)N * TL * a.B;
   ProfScope ps(prof, "spectral_dual", CH * vox * 20.0, 2.0 * CH * 2.0 * TL * vox, st);
-  k_dct_tc<CH><<<(unsigned)grid, CTA_T, SMEM, st>>>(a);
+  launch_chain(k_dct_tc<CH>, (unsigned)grid, CTA_T, SMEM, st, a);
   return cudaGetLastError();
 }
 

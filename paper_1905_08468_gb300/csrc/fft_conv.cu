@@ -17,6 +17,7 @@
 
 #include "fft.cuh"
 #include "fft32.cuh"
+#include "chain.cuh"
 #include "kernels.h"
 
 namespace muffin {
@@ -48,6 +49,7 @@ k_rows_fwd(const float *__restrict__ x, float2 *__restrict__ S,
   const int y0 = blockIdx.x * 2 * nq;
   float2 *d = sm2, *tws = sm2 + nq * pitch;
   load_tw(tws, tw, tlen);
+  chain_enter();
   // element u of the thread is i = tid + 256 u of the [nq][n] row pairs:
   // pair tid / n + 256 u / n, column tid % n + (256 u) % n, so every index
   // is a per-thread base plus a compile-time offset
@@ -95,6 +97,7 @@ k_cols(float2 *__restrict__ S, const float *__restrict__ kspec, int L,
   const int ncol = min(CB, nh - k0);
   float2 *d = sm2, *tws = sm2 + CB * pitch;
   load_tw(tws, tw, tlen);
+  chain_enter();
   // element u of the thread is i = tid + 256 u of the CTA's [CB][n] block:
   // column c0 + 256 u / n, row tid % n + (256 u) % n (see k_rows_fwd)
   const int tid = threadIdx.x;
@@ -147,6 +150,7 @@ k_rows_inv(const float2 *__restrict__ S, float *__restrict__ g,
   const int y0 = blockIdx.x * 2 * nq;
   float2 *d = sm2, *tws = sm2 + nq * pitch;
   load_tw(tws, tw, tlen);
+  chain_enter();
   const float4 *Si = reinterpret_cast<const float4 *>(S + (size_t)img * nh * n);
   for (int i = threadIdx.x; i < nh * nq; i += blockDim.x) {
     const int k = i / nq, q = i - k * nq;
@@ -436,17 +440,17 @@ cudaError_t gradient_n(const float *x, float *g, const float *b, float2 *S,
     {
       ProfScope ps(prof, "grad_rows_fwd", nimg * (img * 4.0 + spec),
                    nimg * (n / 2.0) * fft, st);
-      k_rows_fwd<NN, RMAX><<<dim3(n / RB, nimg), kThreads, smr, st>>>(x, S, tw, tlen, i0);
+      launch_chain(k_rows_fwd<NN, RMAX>, dim3(n / RB, nimg), kThreads, smr, st, x, S, tw, tlen, i0);
     }
     {
       ProfScope ps(prof, "grad_cols", nimg * 2.0 * spec + (double)nimg * nh * n * 4.0,
                    nimg * (double)nh * 2.0 * fft, st);
-      k_cols<NN, RMAX><<<dim3((nh + CB - 1) / CB, nimg), kThreads, smc, st>>>(S, kspec, L, tw, tlen, i0);
+      launch_chain(k_cols<NN, RMAX>, dim3((nh + CB - 1) / CB, nimg), kThreads, smc, st, S, kspec, L, tw, tlen, i0);
     }
     {
       ProfScope ps(prof, "grad_rows_inv", nimg * (spec + img * 4.0) + nb * img * 4.0,
                    nimg * (n / 2.0) * fft, st);
-      k_rows_inv<NN, RMAX><<<dim3(n / RB, nimg), kThreads, smr, st>>>(S, g, b, L, tw, tlen, i0);
+      launch_chain(k_rows_inv<NN, RMAX>, dim3(n / RB, nimg), kThreads, smr, st, S, g, b, L, tw, tlen, i0);
     }
   }
   return cudaGetLastError();

@@ -33,6 +33,7 @@
 
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "kernels.h"
 
 namespace muffin {
@@ -115,6 +116,7 @@ __device__ __forceinline__ void prefetch_tile(const float *img, unsigned n, unsi
 // 1 + blockIdx.z
 template <int MODE, int D, bool LAST, bool DERIV>
 __global__ void __launch_bounds__(INT, 3) k_iuwt_ana(IuwtArgs a) {
+  chain_enter();
   __shared__ float vs[IY * VP];
   const unsigned n = a.n, nm = n - 1;
   const int l = blockIdx.y, c = DERIV ? 1 + blockIdx.z : 0, tid = threadIdx.x;
@@ -209,6 +211,7 @@ __global__ void __launch_bounds__(INT, 3) k_iuwt_ana(IuwtArgs a) {
 // prox, chain 0 or chains 1 + blockIdx.z.
 template <int MODE, int D, bool TOP, bool DERIV>
 __global__ void __launch_bounds__(INT, 3) k_iuwt_syn(IuwtArgs a) {
+  chain_enter();
   __shared__ float vs[IY * VP];
   const unsigned n = a.n, nm = n - 1;
   const int l = blockIdx.y, c = (DERIV ? 1 : 0) + blockIdx.z, tid = threadIdx.x;
@@ -333,11 +336,11 @@ template <int CH, int MODE, int D>
 void launch_ana_d(const IuwtArgs &a, cudaStream_t st) {
   const dim3 g(itiles(a.n), a.L), g2(itiles(a.n), a.L, 2);
   if (a.j == a.J - 1) {
-    k_iuwt_ana<MODE, D, true, false><<<g, INT, 0, st>>>(a);
-    if constexpr (CH == 3) k_iuwt_ana<MODE, D, true, true><<<g2, INT, 0, st>>>(a);
+    launch_chain(k_iuwt_ana<MODE, D, true, false>, g, INT, 0, st, a);
+    if constexpr (CH == 3) launch_chain(k_iuwt_ana<MODE, D, true, true>, g2, INT, 0, st, a);
   } else {
-    k_iuwt_ana<MODE, D, false, false><<<g, INT, 0, st>>>(a);
-    if constexpr (CH == 3) k_iuwt_ana<MODE, D, false, true><<<g2, INT, 0, st>>>(a);
+    launch_chain(k_iuwt_ana<MODE, D, false, false>, g, INT, 0, st, a);
+    if constexpr (CH == 3) launch_chain(k_iuwt_ana<MODE, D, false, true>, g2, INT, 0, st, a);
   }
 }
 
@@ -345,11 +348,11 @@ template <int CH, int MODE, int D>
 void launch_syn_d(const IuwtArgs &a, cudaStream_t st) {
   const bool top = a.j == a.J - 1;
   const dim3 g(itiles(a.n), a.L, D > 1 ? CH : 1), g2(itiles(a.n), a.L, 2);
-  if (top) k_iuwt_syn<MODE, D, true, false><<<g, INT, 0, st>>>(a);
-  else k_iuwt_syn<MODE, D, false, false><<<g, INT, 0, st>>>(a);
+  if (top) launch_chain(k_iuwt_syn<MODE, D, true, false>, g, INT, 0, st, a);
+  else launch_chain(k_iuwt_syn<MODE, D, false, false>, g, INT, 0, st, a);
   if constexpr (CH == 3 && D == 1) {
-    if (top) k_iuwt_syn<MODE, D, true, true><<<g2, INT, 0, st>>>(a);
-    else k_iuwt_syn<MODE, D, false, true><<<g2, INT, 0, st>>>(a);
+    if (top) launch_chain(k_iuwt_syn<MODE, D, true, true>, g2, INT, 0, st, a);
+    else launch_chain(k_iuwt_syn<MODE, D, false, true>, g2, INT, 0, st, a);
   }
 }
 

@@ -37,6 +37,7 @@
 // (Algorithm 4 has its inhomogeneous terms in the spectral step).
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "kernels.h"
 #include "wavelet.h"
 
@@ -293,6 +294,7 @@ __device__ __forceinline__ void ana_emit_step(const AnaArgs &a, int l, int bb, i
 // Small levels (ana_cols.cu serves the rest).
 template <int CH, int MODE, bool LEVEL1>
 __global__ void __launch_bounds__(NT, 4) k_ana(AnaArgs a) {
+  chain_enter();
   extern __shared__ float2 smem2[];
   float2 *in_s = smem2;                     // [CH][A_RP][A_IP] row pairs
   float2 *lohi = in_s + CH * A_RP * A_IP;   // [A_RP][A_LP] lo, then hi
@@ -635,6 +637,7 @@ __device__ __forceinline__ void syn_dispatch(int p, const float *cf, float *lo,
 // which is faster depends on the shape, so the plan's tuner picks one.
 template <int CH, int MODE, bool LEVEL1, bool PACKED>
 __global__ void __launch_bounds__(NT, 4) k_syn(SynArgs a) {
+  chain_enter();
   constexpr int ROWS = PACKED ? 2 : 1;   // pixel rows per thread
   constexpr int NO = PACKED ? 2 * QXP : 2 * QXS;   // pixels per row
   extern __shared__ float smem[];
@@ -806,6 +809,7 @@ __global__ void __launch_bounds__(NT, 4) k_syn(SynArgs a) {
 // ------------------------------------------------------------ J = 0 (identity bases)
 template <int CH, int MODE>
 __global__ void k_syn0(SynArgs a) {
+  chain_enter();
   const size_t NN = (size_t)a.n * a.n;
   const size_t tot = (size_t)a.L * NN;
   const size_t US = (size_t)a.L * a.K * NN, CS = (size_t)a.L * NN;
@@ -845,6 +849,7 @@ __global__ void k_syn0(SynArgs a) {
 
 template <int CH, int MODE>
 __global__ void k_ana0(AnaArgs a) {
+  chain_enter();
   const size_t NN = (size_t)a.n * a.n;
   const size_t tot = (size_t)a.L * NN, CS = (size_t)a.L * NN;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < tot;
@@ -885,7 +890,7 @@ cudaError_t launch_ana(const AnaArgs &a, int nblk_y, cudaStream_t st) {
                          (int)smem);
     attr = true;
   }
-  k_ana<CH, MODE, L1><<<dim3(tiles(a.M >> 1), nblk_y), NT, smem, st>>>(a);
+  launch_chain(k_ana<CH, MODE, L1>, dim3(tiles(a.M >> 1), nblk_y), NT, smem, st, a);
   return cudaGetLastError();
 }
 
@@ -901,7 +906,7 @@ cudaError_t launch_syn_v(const SynArgs &a, int nblk_y, cudaStream_t st) {
   // K C steps in CTAs of their own (64 x 64 x 8: 12.6 and 12.4 -> 6.9 and 6.4 us;
   // 256 x 256 x 32, level 3: 13.2 -> 8.7 us, three chains 28 -> 14.6)
   const int nt = tiles(a.M >> 1), nz = !L1 && nt * nblk_y < 304 ? a.K * CH : 1;
-  k_syn<CH, MODE, L1, PACKED><<<dim3(nt, nblk_y, nz), NT, syn_smem(CH), st>>>(a);
+  launch_chain(k_syn<CH, MODE, L1, PACKED>, dim3(nt, nblk_y, nz), NT, syn_smem(CH), st, a);
   return cudaGetLastError();
 }
 
@@ -928,7 +933,7 @@ cudaError_t synthesis_all(const WaveArgs &w, const SynArgs &base, cudaStream_t s
   if (w.J == 0) {
     a.M = w.n;
     ProfScope ps(w.prof, "syn_identity_prox", (double)CH * w.L * w.n * w.n * 4.0 * (w.K + 4), 0.0, st);
-    k_syn0<CH, MODE><<<grid_elem((size_t)w.L * w.n * w.n), 256, 0, st>>>(a);
+    launch_chain(k_syn0<CH, MODE>, grid_elem((size_t)w.L * w.n * w.n), 256, 0, st, a);
     return cudaGetLastError();
   }
   cudaError_t e = cudaSuccess;
@@ -953,7 +958,7 @@ cudaError_t analysis_all(const WaveArgs &w, const AnaArgs &base, cudaStream_t st
   if (w.J == 0) {
     a.M = w.n;
     ProfScope ps(w.prof, "ana_identity_dual", (double)CH * w.L * w.n * w.n * 4.0 * (2 * w.K + 2), 0.0, st);
-    k_ana0<CH, MODE><<<grid_elem((size_t)w.L * w.n * w.n), 256, 0, st>>>(a);
+    launch_chain(k_ana0<CH, MODE>, grid_elem((size_t)w.L * w.n * w.n), 256, 0, st, a);
     return cudaGetLastError();
   }
   cudaError_t e = cudaSuccess;
