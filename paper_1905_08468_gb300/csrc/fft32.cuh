@@ -175,6 +175,94 @@ __device__ __forceinline__ void fft_stages(float2 *d, int pitch, int nthr,
   }
 }
 
+// The first stage (NS = 1, no twiddles) of sequences whose elements the caller
+// has in registers: v[g * R + r] holds element j + r N / R of sequence s, with
+// w = tid + g nthr = s N / R + j.  Leaves the stage's outputs in shared memory.
+template <int N, int R, int VPT, bool INV>
+__device__ __forceinline__ void fft_first(float2 (&v)[VPT], float2 *d, int pitch, int nthr) {
+  constexpr int G = VPT / R, q = N / R;
+  if (threadIdx.x < nthr) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      dftR<R, INV>(v + g * R);
+      const int w = threadIdx.x + g * nthr;
+      float2 *dst = d + (w / q) * pitch;
+      const int o = (w % q) * R;
+#pragma unroll
+      for (int r = 0; r < R; ++r) dst[fpad(o + r)] = v[g * R + out_slot<R>(r)];
+    }
+  }
+  __syncthreads();
+}
+
+// The last stage (NS R = N), left in registers: v[g * R + out_slot<R>(r)] is
+// element j + r NS of sequence s, w = tid + g nthr = s NS + j.
+template <int N, int NS, int R, int VPT, bool INV>
+__device__ __forceinline__ void fft_last(float2 (&v)[VPT], const float2 *d, int pitch, int nthr,
+                                         const float2 *tw) {
+  static_assert(NS * R == N, "the last stage");
+  constexpr int G = VPT / R;
+  if (threadIdx.x < nthr) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const int w = threadIdx.x + g * nthr, j = w % NS;
+      const float2 *src = d + (w / NS) * pitch;
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[g * R + r] = src[fpad(j + r * NS)];
+      if (NS > 1) {
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[g * R + r] = twid<INV>(v[g * R + r], tw[(r - 1) * NS + j]);
+      }
+      dftR<R, INV>(v + g * R);
+    }
+  }
+}
+
+// length before the last stage of the plan
+__host__ __device__ constexpr int fft_last_ns(int N, int rmax) {
+  int ns = 1;
+  while (N / ns > rmax) ns *= rmax;
+  return ns;
+}
+
+// the stages from NS up to (not with) the last one
+template <int N, int NS, bool INV, int RMAX>
+__device__ __forceinline__ const float2 *fft_middle(float2 *d, int pitch, int nthr,
+                                                    const float2 *tw) {
+  if constexpr (NS < fft_last_ns(N, RMAX)) {
+    fft_stage<N, NS, RMAX, fft_vpt(N), INV>(d, pitch, nthr, tw);
+    return fft_middle<N, NS * RMAX, INV, RMAX>(d, pitch, nthr,
+                                               tw + (NS > 1 ? (RMAX - 1) * NS : 0));
+  }
+  return tw;
+}
+
+// ---- in-place plan of the column pass (N >= 64): decimation in frequency with
+// radices 16, 16 (N > 256) and a last one of 2 .. 16, backwards by the mirrored
+// stages, so that the last forward and the first inverse stage meet in registers
+// and no stage reorders.  Position p of a column then holds frequency
+// cols_freq(p) between the two.
+__host__ __device__ constexpr int cols_last_radix(int N) { return N > 256 ? N / 256 : N / 16; }
+__host__ __device__ constexpr int cols_pos(int f, int N) {
+  return N > 256 ? ((f & 15) * 16 + ((f >> 4) & 15)) * cols_last_radix(N) + (f >> 8)
+                 : (f & 15) * cols_last_radix(N) + (f >> 4);
+}
+// twiddles exp(-2 pi i t k / len), k = 1 .. 15, at [(k - 1) len / 16 + t] for len = N
+// and (N > 256) len = N / 16
+__host__ __device__ constexpr int cols_table_len(int N) {
+  return N < 64 ? 1 : 15 * (N / 16) + (N > 256 ? 15 * (N / 256) : 0);
+}
+inline void cols_tables(int N, float2 *tab) {
+  const double pi = 3.14159265358979323846;
+  if (N < 64) { tab[0] = make_float2(1.f, 0.f); return; }
+  for (int len = N, off = 0; len == N || (N > 256 && len == N / 16); off += 15 * (len / 16), len /= 16)
+    for (int k = 1; k < 16; ++k)
+      for (int t = 0; t < len / 16; ++t) {
+        const double a = -2.0 * pi * (double)t * k / (double)len;
+        tab[off + (k - 1) * (len / 16) + t] = make_float2((float)std::cos(a), (float)std::sin(a));
+      }
+}
+
 // In-place transform of nb sequences (sequence s at d + s * pitch, padded
 // layout).  Needs nb * N / fft_vpt(N) <= blockDim.x.  Caller syncs before.
 template <int N, bool INV, int RMAX = 16>

@@ -31,6 +31,16 @@ __host__ __device__ constexpr int seqs_per_cta(int n) { return kThreads * fft_vp
 // complex (row-pair) sequences per CTA of the row passes: 2 * nq real rows
 __host__ __device__ constexpr int row_pairs(int n) { return seqs_per_cta(n) < n / 2 ? seqs_per_cta(n) : n / 2; }
 
+// Shared-memory distance of the row passes' sequences: the split into (and the
+// rebuild from) half spectra walks the pairs of a bin first, so the pairs of 16
+// consecutive threads have to start in different banks (n + n / 16 is a multiple
+// of 16 from 256 on, and 4-, 8- and 16-way conflicts bound the passes: 96 images
+// of 256 x 256, forward 28.2 -> 17.3 us, inverse 26.9 -> 17.6; 192 images of 1024 x
+// 1024, 391 -> 357 and 473 -> 454).
+__host__ __device__ constexpr int row_pitch(int n) {
+  return n + (n >> 4) + (row_pairs(n) >= 16 ? 1 : 16 / row_pairs(n));
+}
+
 // stage the twiddle tables (tlen entries) into shared memory
 __device__ __forceinline__ void load_tw(float2 *dst, const float2 *__restrict__ src, int tlen) {
   for (int i = threadIdx.x; i < tlen; i += blockDim.x) dst[i] = src[i];
@@ -42,7 +52,7 @@ k_rows_fwd(const float *__restrict__ x, float2 *__restrict__ S,
            const float2 *__restrict__ tw, int tlen, int img0) {
   // sizes are compile-time so that the index splits below are shifts
   constexpr int n = NN, nq = row_pairs(NN), nh = (NN >> 1) + 1;
-  constexpr int pitch = n + (n >> 4);
+  constexpr int pitch = row_pitch(NN);
   extern __shared__ float2 sm2[];
   const int img = blockIdx.y;           // image of the chunk (its spectrum in S)
   const int gimg = img0 + img;          // image of the cube
@@ -50,27 +60,22 @@ k_rows_fwd(const float *__restrict__ x, float2 *__restrict__ S,
   float2 *d = sm2, *tws = sm2 + nq * pitch;
   load_tw(tws, tw, tlen);
   chain_enter();
-  // element u of the thread is i = tid + 256 u of the [nq][n] row pairs:
-  // pair tid / n + 256 u / n, column tid % n + (256 u) % n, so every index
-  // is a per-thread base plus a compile-time offset
-  const int tid = threadIdx.x;
-  const float *xi = x + (size_t)gimg * n * n + (size_t)(y0 + 2 * (tid / n)) * n + tid % n;
-  const int sb = (tid / n) * pitch + fpad(tid % n);
-  constexpr int VPT = fft_vpt(NN);
+  // the first stage straight from the rows: element j + r q of pair s in the
+  // stage's register order (coalesced: consecutive threads, consecutive j)
+  constexpr int VPT = fft_vpt(NN), R = n < RMAX ? n : RMAX, q = n / R;
+  constexpr int nthr = nq * n / VPT;
   float2 v[VPT];
+  if (threadIdx.x < nthr) {
 #pragma unroll
-  for (int u = 0; u < VPT; ++u) {
-    const int q = (kThreads * u) / n, c = (kThreads * u) % n;
-    if (tid + u * kThreads < nq * n)
-      v[u] = make_float2(xi[2 * q * n + c], xi[(2 * q + 1) * n + c]);
-  }
+    for (int g = 0; g < VPT / R; ++g) {
+      const int w = threadIdx.x + g * nthr;
+      const float *xi = x + (size_t)gimg * n * n + (size_t)(y0 + 2 * (w / q)) * n + w % q;
 #pragma unroll
-  for (int u = 0; u < VPT; ++u) {
-    const int q = (kThreads * u) / n, c = (kThreads * u) % n;
-    if (tid + u * kThreads < nq * n) d[sb + q * pitch + fpad(c)] = v[u];
+      for (int r = 0; r < R; ++r) v[g * R + r] = make_float2(xi[r * q], xi[n + r * q]);
+    }
   }
-  __syncthreads();
-  fft_inplace<NN, false, RMAX>(d, nq, pitch, tws);
+  fft_first<NN, R, VPT, false>(v, d, pitch, nthr);
+  fft_stages<NN, R, false, RMAX>(d, pitch, nthr, tws);
   float4 *Si = reinterpret_cast<float4 *>(S + (size_t)img * nh * n);
   for (int i = threadIdx.x; i < nh * nq; i += blockDim.x) {
     const int k = i / nq, q = i - k * nq;
@@ -138,13 +143,120 @@ k_cols(float2 *__restrict__ S, const float *__restrict__ kspec, int L,
       Si[kThreads * u] = d[sb + ((kThreads * u) / n) * pitch + fpad((kThreads * u) % n)];
 }
 
+// The column pass from 64 rows on.  What bounds the Stockham form above is the
+// shared-memory pipe (76 percent busy at 31 percent of the DRAM rate): an element
+// crosses it 16 times and the CTA meets at 16 barriers.  Here (in-place plan of
+// fft32.cuh) it crosses 8 times and meets at 4, columns come from and go to
+// global memory in registers, and the multipliers, stored in the order of the
+// positions, are read as the last stage holds them.  192 images of 1024 x 1024:
+// 560 -> 413 us (4.9 TB/s); 32 images of 256 x 256: 16.3 -> 10.8 us.
+template <int NN>
+__global__ void __launch_bounds__(kThreads, 3)
+k_cols_dif(float2 *__restrict__ S, const float *__restrict__ kspec, int L,
+           const float2 *__restrict__ tw, int img0) {
+  constexpr int n = NN, nh = (NN >> 1) + 1, CB = seqs_per_cta(NN), pitch = n + (n >> 4);
+  constexpr int T = n / 16, M = n / 16, RL = cols_last_radix(n), GL = 16 / RL;
+  constexpr bool three = n > 256;
+  constexpr int tlen = cols_table_len(n);
+  extern __shared__ float2 sm2[];
+  float2 *tw1 = sm2 + CB * pitch, *tw2 = tw1 + 15 * T;
+  load_tw(tw1, tw, tlen);
+  chain_enter();
+  const int img = blockIdx.y, band = (img0 + img) % L;
+  const int k0 = blockIdx.x * CB, c = threadIdx.x / T, t = threadIdx.x % T;
+  const bool act = c < CB && k0 + c < nh;
+  float2 *d = sm2 + c * pitch;
+  float2 *Si = S + ((size_t)img * nh + k0 + c) * n + t;
+  float2 v[16];
+  float kr[16];
+  if (act) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = Si[r * T];
+    const float *Ki = kspec + ((size_t)band * nh + k0 + c) * n;
+#pragma unroll
+    for (int g = 0; g < GL; ++g)
+#pragma unroll
+      for (int e = 0; e < RL; e += (RL < 4 ? 2 : 4)) {
+        if constexpr (RL < 4) {
+          const float2 k2 = __ldg(reinterpret_cast<const float2 *>(Ki + (t + g * T) * RL + e));
+          kr[g * RL + e] = k2.x; kr[g * RL + e + 1] = k2.y;
+        } else {
+          const float4 k4 = __ldg(reinterpret_cast<const float4 *>(Ki + (t + g * T) * RL + e));
+          kr[g * RL + e] = k4.x; kr[g * RL + e + 1] = k4.y;
+          kr[g * RL + e + 2] = k4.z; kr[g * RL + e + 3] = k4.w;
+        }
+      }
+  }
+  __syncthreads();                       // the tables
+  const int t2 = t % (three ? M / 16 : 1), k1 = t / (three ? M / 16 : 1);
+  if (act) {
+    dft16<false>(v);
+    d[fpad(t)] = v[0];
+#pragma unroll
+    for (int r = 1; r < 16; ++r) d[fpad(r * M + t)] = cmul(v[out_slot<16>(r)], tw1[(r - 1) * T + t]);
+  }
+  __syncthreads();
+  if constexpr (three) {
+    if (act) {
+      float2 *e = d + fpad(k1 * M);      // M is a multiple of 16
+#pragma unroll
+      for (int r = 0; r < 16; ++r) v[r] = e[fpad(t2 + r * (M / 16))];
+      dft16<false>(v);
+      e[t2] = v[0];
+#pragma unroll
+      for (int r = 1; r < 16; ++r)
+        e[fpad(r * (M / 16) + t2)] = cmul(v[out_slot<16>(r)], tw2[(r - 1) * (M / 16) + t2]);
+    }
+    __syncthreads();
+  }
+  if (act) {
+#pragma unroll
+    for (int g = 0; g < GL; ++g) {
+      float2 w[RL], u[RL];
+#pragma unroll
+      for (int e = 0; e < RL; ++e) w[e] = d[fpad((t + g * T) * RL + e)];
+      dftR<RL, false>(w);
+#pragma unroll
+      for (int e = 0; e < RL; ++e) {
+        const float2 z = w[out_slot<RL>(e)];
+        u[e] = make_float2(z.x * kr[g * RL + e], z.y * kr[g * RL + e]);
+      }
+      dftR<RL, true>(u);
+#pragma unroll
+      for (int e = 0; e < RL; ++e) d[fpad((t + g * T) * RL + e)] = u[out_slot<RL>(e)];
+    }
+  }
+  __syncthreads();
+  if constexpr (three) {
+    if (act) {
+      float2 *e = d + fpad(k1 * M);
+      v[0] = e[t2];
+#pragma unroll
+      for (int r = 1; r < 16; ++r)
+        v[r] = cmulc(e[fpad(r * (M / 16) + t2)], tw2[(r - 1) * (M / 16) + t2]);
+      dft16<true>(v);
+#pragma unroll
+      for (int r = 0; r < 16; ++r) e[fpad(t2 + r * (M / 16))] = v[out_slot<16>(r)];
+    }
+    __syncthreads();
+  }
+  if (act) {
+    v[0] = d[fpad(t)];
+#pragma unroll
+    for (int r = 1; r < 16; ++r) v[r] = cmulc(d[fpad(r * M + t)], tw1[(r - 1) * T + t]);
+    dft16<true>(v);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) Si[r * T] = v[out_slot<16>(r)];
+  }
+}
+
 template <int NN, int RMAX>
 __global__ void __launch_bounds__(kThreads)
-k_rows_inv(const float2 *__restrict__ S, float *__restrict__ g,
+k_rows_inv(const float2 *__restrict__ S, float *__restrict__ g_out,
            const float *__restrict__ bdata, int L,
            const float2 *__restrict__ tw, int tlen, int img0) {
   constexpr int n = NN, nq = row_pairs(NN), nh = (NN >> 1) + 1, half = NN >> 1;
-  constexpr int pitch = n + (n >> 4);
+  constexpr int pitch = row_pitch(NN);
   extern __shared__ float2 sm2[];
   const int img = blockIdx.y, gimg = img0 + img, band = gimg % L;
   const int y0 = blockIdx.x * 2 * nq;
@@ -161,27 +273,55 @@ k_rows_inv(const float2 *__restrict__ S, float *__restrict__ g,
       d[q * pitch + fpad(n - k)] = make_float2(v.x + v.w, v.z - v.y);  // conj Xa + i conj Xb
   }
   __syncthreads();
-  fft_inplace<NN, true, RMAX>(d, nq, pitch, tws);
   const bool sub = (bdata != nullptr) && (gimg < L);
-  // element u of the thread: row pair tid / n + 256 u / n (see k_rows_fwd)
-  const int tid = threadIdx.x;
-  const size_t o0 = (size_t)(y0 + 2 * (tid / n)) * n + tid % n;
-  float *gi = g + (size_t)gimg * n * n + o0;
-  const float *bi = sub ? bdata + (size_t)band * n * n + o0 : nullptr;
-  const int sb = (tid / n) * pitch + fpad(tid % n);
-  constexpr int VPT = fft_vpt(NN);
+  constexpr int VPT = fft_vpt(NN), NS = fft_last_ns(n, RMAX), R = n / NS;
+  constexpr int nthr = nq * n / VPT;
+  if constexpr (NS >= 32) {
+    // the last stage's registers go straight to the rows (element j + r NS of pair
+    // s: whole lines a warp)
+    const float2 *twl = fft_middle<NN, 1, true, RMAX>(d, pitch, nthr, tws);
+    float2 v[VPT];
+    fft_last<NN, NS, R, VPT, true>(v, d, pitch, nthr, twl);
+    if (threadIdx.x >= nthr) return;
 #pragma unroll
-  for (int u = 0; u < VPT; ++u) {
-    if (tid + u * kThreads >= nq * n) continue;
-    const int q = (kThreads * u) / n, c = (kThreads * u) % n;
-    const float2 z = d[sb + q * pitch + fpad(c)];
-    float v0 = z.x, v1 = z.y;
-    if (sub) {
-      v0 -= __ldg(bi + 2 * q * n + c);
-      v1 -= __ldg(bi + (2 * q + 1) * n + c);
+    for (int g = 0; g < VPT / R; ++g) {
+      const int w = threadIdx.x + g * nthr;
+      const size_t o0 = (size_t)(y0 + 2 * (w / NS)) * n + w % NS;
+      float *gi = g_out + (size_t)gimg * n * n + o0;
+      const float *bi = sub ? bdata + (size_t)band * n * n + o0 : nullptr;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float2 z = v[g * R + out_slot<R>(r)];
+        float v0 = z.x, v1 = z.y;
+        if (sub) {
+          v0 -= __ldg(bi + r * NS);
+          v1 -= __ldg(bi + n + r * NS);
+        }
+        gi[r * NS] = v0;
+        gi[n + r * NS] = v1;
+      }
     }
-    gi[2 * q * n + c] = v0;
-    gi[(2 * q + 1) * n + c] = v1;
+  } else {
+    fft_inplace<NN, true, RMAX>(d, nq, pitch, tws);
+    // element u of the thread: row pair tid / n + 256 u / n, column tid % n + ...
+    const int tid = threadIdx.x;
+    const size_t o0 = (size_t)(y0 + 2 * (tid / n)) * n + tid % n;
+    float *gi = g_out + (size_t)gimg * n * n + o0;
+    const float *bi = sub ? bdata + (size_t)band * n * n + o0 : nullptr;
+    const int sb = (tid / n) * pitch + fpad(tid % n);
+#pragma unroll
+    for (int u = 0; u < VPT; ++u) {
+      if (tid + u * kThreads >= nq * n) continue;
+      const int q = (kThreads * u) / n, c = (kThreads * u) % n;
+      const float2 z = d[sb + q * pitch + fpad(c)];
+      float v0 = z.x, v1 = z.y;
+      if (sub) {
+        v0 -= __ldg(bi + 2 * q * n + c);
+        v1 -= __ldg(bi + (2 * q + 1) * n + c);
+      }
+      gi[2 * q * n + c] = v0;
+      gi[(2 * q + 1) * n + c] = v1;
+    }
   }
 }
 
@@ -373,7 +513,8 @@ __global__ void k_c64_real_to_f32(const double2 *__restrict__ in,
     out[i] = (float)(in[i].x * scale);
 }
 
-// grid (n / 2 + 1, L); max_bits[l]: the largest |hh|^2 of the band (bits of a
+// grid (n / 2 + 1, L); rows in the order of the column pass's positions;
+// max_bits[l]: the largest |hh|^2 of the band (bits of a
 // double >= 0, which order as integers, and above them NaN; the other half of a
 // spectrum holds the conjugates)
 __global__ void k_make_kspec(const double2 *__restrict__ hh, float *__restrict__ kspec,
@@ -385,7 +526,7 @@ __global__ void k_make_kspec(const double2 *__restrict__ hh, float *__restrict__
   for (int ky = threadIdx.x; ky < n; ky += blockDim.x) {
     const double v = h[ky].x * h[ky].x + h[ky].y * h[ky].y;
     m = max(m, (unsigned long long)__double_as_longlong(fabs(v)));
-    k[ky] = (float)(v * scale);
+    k[n < 64 ? ky : cols_pos(ky, n)] = (float)(v * scale);
   }
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
@@ -407,7 +548,7 @@ inline int grid_for(size_t count) {
 
 template <int NN, int RMAX>
 cudaError_t gradient_n(const float *x, float *g, const float *b, float2 *S,
-                       const float *kspec, const float2 *tw, int L, int C,
+                       const float *kspec, const float2 *tw, const float2 *twc, int L, int C,
                        cudaStream_t st, Prof *prof, int chunk) {
   constexpr int n = NN;
   const int ntot = C * L;
@@ -416,13 +557,16 @@ cudaError_t gradient_n(const float *x, float *g, const float *b, float2 *S,
   const int nh = (n >> 1) + 1;
   const int pitch = n + (n >> 4);
   const int tlen = fft_table_len(n, RMAX);
-  const size_t smr = ((size_t)(RB / 2) * pitch + tlen) * sizeof(float2);
-  const size_t smc = ((size_t)CB * pitch + tlen) * sizeof(float2);
+  const size_t smr = ((size_t)(RB / 2) * row_pitch(n) + tlen) * sizeof(float2);
+  const size_t smc = ((size_t)CB * pitch + (n >= 64 ? cols_table_len(n) : tlen)) * sizeof(float2);
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_rows_fwd<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_rows_inv<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_cols<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if constexpr (NN >= 64)
+      cudaFuncSetAttribute(k_cols_dif<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    else
+      cudaFuncSetAttribute(k_cols<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr = true;
   }
   const double img = (double)n * n, spec = (double)nh * n * 8.0;
@@ -445,7 +589,9 @@ cudaError_t gradient_n(const float *x, float *g, const float *b, float2 *S,
     {
       ProfScope ps(prof, "grad_cols", nimg * 2.0 * spec + (double)nimg * nh * n * 4.0,
                    nimg * (double)nh * 2.0 * fft, st);
-      launch_chain(k_cols<NN, RMAX>, dim3((nh + CB - 1) / CB, nimg), kThreads, smc, st, S, kspec, L, tw, tlen, i0);
+      const dim3 grid((nh + CB - 1) / CB, nimg);
+      if constexpr (NN >= 64) launch_chain(k_cols_dif<NN>, grid, kThreads, smc, st, S, kspec, L, twc, i0);
+      else launch_chain(k_cols<NN, RMAX>, grid, kThreads, smc, st, S, kspec, L, tw, tlen, i0);
     }
     {
       ProfScope ps(prof, "grad_rows_inv", nimg * (spec + img * 4.0) + nb * img * 4.0,
@@ -459,14 +605,14 @@ cudaError_t gradient_n(const float *x, float *g, const float *b, float2 *S,
 }  // namespace
 
 cudaError_t launch_gradient(const float *x, float *g, const float *b,
-                            float2 *S, const float *kspec, const float2 *tw,
+                            float2 *S, const float *kspec, const float2 *tw, const float2 *twc,
                             int n, int L, int C, cudaStream_t st, Prof *prof, int chunk,
                             int radix) {
   const bool r8 = radix == 8 && n >= 64;   // the alternative plan exists from n = 64
 #define MUFFIN_GRAD(NN)                                                                    \
-  return r8 ? gradient_n<NN, 8>(x, g, b, S, kspec, tw, L, C, st, prof, chunk)              \
-            : gradient_n<NN, 16>(x, g, b, S, kspec, tw, L, C, st, prof, chunk)
-#define MUFFIN_GRAD16(NN) return gradient_n<NN, 16>(x, g, b, S, kspec, tw, L, C, st, prof, chunk)
+  return r8 ? gradient_n<NN, 8>(x, g, b, S, kspec, tw, twc, L, C, st, prof, chunk)              \
+            : gradient_n<NN, 16>(x, g, b, S, kspec, tw, twc, L, C, st, prof, chunk)
+#define MUFFIN_GRAD16(NN) return gradient_n<NN, 16>(x, g, b, S, kspec, tw, twc, L, C, st, prof, chunk)
   switch (n) {
     case 2: MUFFIN_GRAD16(2);
     case 4: MUFFIN_GRAD16(4);
@@ -487,6 +633,8 @@ cudaError_t launch_gradient(const float *x, float *g, const float *b,
 
 int fft32_table_len(int n, int radix) { return fft_table_len(n, radix); }
 void fft32_tables(int n, float2 *tab, int radix) { fft_tables(n, tab, radix); }
+int fft32_cols_table_len(int n) { return cols_table_len(n); }
+void fft32_cols_tables(int n, float2 *tab) { cols_tables(n, tab); }
 
 cudaError_t fft2d_c64(double2 *data, double2 *tmp, int n, int nimg,
                       bool inverse, const double2 *tw64, cudaStream_t st) {

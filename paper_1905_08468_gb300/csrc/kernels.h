@@ -98,7 +98,7 @@ int set_last_error_code(int s, const char *msg);
 // radix 16 (default) or 8 (n >= 64): the largest radix of the FFT plan; tw
 // must hold that plan's twiddle tables (fft32_tables with the same radix).
 cudaError_t launch_gradient(const float *x, float *g, const float *b,
-                            float2 *S, const float *kspec, const float2 *tw,
+                            float2 *S, const float *kspec, const float2 *tw, const float2 *twc,
                             int n, int L, int C, cudaStream_t st,
                             Prof *prof = nullptr, int chunk = 0, int radix = 16);
 
@@ -106,6 +106,9 @@ cudaError_t launch_gradient(const float *x, float *g, const float *b,
 // the plan whose largest radix is `radix`.
 int fft32_table_len(int n, int radix = 16);
 void fft32_tables(int n, float2 *tab, int radix = 16);
+// Twiddles of the column pass from 64 rows on (twc above; any radix).
+int fft32_cols_table_len(int n);
+void fft32_cols_tables(int n, float2 *tab);
 
 // FP64 helpers used when a plan or a call is set up.
 // In-place 2D DFT of nimg complex n x n images; inverse is unnormalised.
@@ -131,7 +134,8 @@ cudaError_t convolve_real(const float *x, const ImageStat *stat, const double2 *
 // out = (float)(scale * in.x)
 cudaError_t c64_real_to_f32(const double2 *in, float *out, double scale,
                             size_t count, cudaStream_t st);
-// kspec[l][kx][ky] = |hh[l][kx][ky]|^2 * scale for kx < n/2+1; hmax[l] = the
+// kspec[l][kx][.] = |hh[l][kx][ky]|^2 * scale for kx < n/2+1, in the column pass's
+// order of ky (cols_pos in fft32.cuh; natural below 64 rows); hmax[l] = the
 // largest |hh[l]|^2 (NaN if any is)
 cudaError_t make_kspec(const double2 *hh, float *kspec, double scale, int n,
                        int L, double *hmax, cudaStream_t st);

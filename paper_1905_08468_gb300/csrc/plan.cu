@@ -231,7 +231,7 @@ muffin_status iterate_kernels(muffin_plan P, const Group &g, int c0, int c1,
     d.alpha += (size_t)c0 * P->N;
     d.sc += c0;
   }
-  CK(launch_gradient(h.x, h.g, h.b, S, kspec, P->tw(), P->n, Lv, g.C, st,
+  CK(launch_gradient(h.x, h.g, h.b, S, kspec, P->tw(), P->twc(), P->n, Lv, g.C, st,
                      P->pp(), P->grad_chunk, P->fft_radix));
   w.L = Lv;
   w.scratch = ll;
@@ -288,7 +288,7 @@ muffin_status iterate_groups(muffin_plan P) {
   }
   Group *gs[2] = {&P->grp[0], &P->grp[1]};
   for (Group *g : gs)
-    CK(launch_gradient(g->x, g->g, g->b, P->S, P->kspec, P->tw(), P->n, P->Lt, g->C, P->ws,
+    CK(launch_gradient(g->x, g->g, g->b, P->S, P->kspec, P->tw(), P->twc(), P->n, P->Lt, g->C, P->ws,
                        P->pp(), P->grad_chunk, P->fft_radix));
   for (Group *g : gs) CK(wavelet_synthesis_prox(P->wave(g->C), *g, P->p.positivity, P->ws));
   for (Group *g : gs) CK(wavelet_analysis_dual(P->wave(g->C), *g, P->ws));
@@ -382,7 +382,8 @@ muffin_status plan_alloc_init(muffin_plan P, const float *alpha, const float *be
   CK(P->alloc(&P->w64b, NL));
   CK(P->alloc(&P->kspec, (size_t)Lt * nh * n));
   P->tw_len16 = fft32_table_len(n, 16);
-  CK(P->alloc(&P->tw32, (size_t)P->tw_len16 + fft32_table_len(n, 8)));
+  const size_t tw_len = (size_t)P->tw_len16 + fft32_table_len(n, 8);
+  CK(P->alloc(&P->tw32, tw_len + fft32_cols_table_len(n)));
   CK(P->alloc(&P->tw64, (size_t)n));
   const size_t LL2 = (size_t)P->Lp * P->Lp;
   CK(P->alloc(&P->chi, LL2));
@@ -454,9 +455,10 @@ muffin_status plan_alloc_init(muffin_plan P, const float *alpha, const float *be
     tdd[k] = make_float4(ch, (float)(t64[k].x - ch), sh, (float)(t64[k].y - sh));
   }
   CK(cudaMemcpyAsync(P->twdd, tdd.data(), n * sizeof(float4), cudaMemcpyHostToDevice, P->ws));
-  std::vector<float2> t32((size_t)P->tw_len16 + fft32_table_len(n, 8));
+  std::vector<float2> t32(tw_len + fft32_cols_table_len(n));
   fft32_tables(n, t32.data(), 16);
   fft32_tables(n, t32.data() + P->tw_len16, 8);
+  fft32_cols_tables(n, t32.data() + tw_len);
   CK(cudaMemcpyAsync(P->tw32, t32.data(), t32.size() * sizeof(float2), cudaMemcpyHostToDevice, P->ws));
   CK(cudaMemcpyAsync(P->tw64, t64.data(), n * sizeof(double2), cudaMemcpyHostToDevice, P->ws));
 
@@ -534,7 +536,7 @@ muffin_status window_end(muffin_plan P, const muffin_sure_params *sp) {
   Group &g = P->grp[0];
   Group g0 = g;
   g0.C = 1;
-  CK(launch_gradient(g0.x, g0.g, g0.b, P->S, P->kspec, P->tw(), P->n, P->Lt, 1, P->ws,
+  CK(launch_gradient(g0.x, g0.g, g0.b, P->S, P->kspec, P->tw(), P->twc(), P->n, P->Lt, 1, P->ws,
                      P->pp(), P->grad_chunk, P->fft_radix));
   SureStatsArgs sa{};
   sa.grad = g.g; sa.x = g.x; sa.xb = P->grp[1].x; sa.b = P->b; sa.htd = P->htd;
@@ -833,7 +835,7 @@ size_t estimate_bytes(const muffin_params *p) {
   if (p->dictionary == 1) ll = 2 * C * Lt * N;
   else
     for (int j = 1; j < p->levels; ++j) ll += C * Lt * K * (n >> j) * (n >> j);
-  size_t b = 3 * NL * 16 + Lt * nh * n * 4 + (size_t)(fft32_table_len((int)n, 16) + fft32_table_len((int)n, 8)) * 8 + n * 16 +
+  size_t b = 3 * NL * 16 + Lt * nh * n * 4 + (size_t)(fft32_table_len((int)n, 16) + fft32_table_len((int)n, 8) + fft32_cols_table_len((int)n)) * 8 + n * 16 +
              4 * Lp * Lp * 4 + (size_t)dct_fold_table_len((int)L) * 4 + B * N * 4 + Lt * 4 + B * sizeof(DevScalars) + B * 32 + 4 + 4 +
              (kRedSure + 65 * Lt + 6 * (Lt > 4096 ? Lt : 4096)) * 8 + Lt * 8 + Lt * sizeof(ImageStat) + Lt * 8 + n * 16 +
              C * Lt * nh * n * 8 + (ll ? ll : 1) * 4 + 3 * NL * 4 +
@@ -1587,7 +1589,7 @@ muffin_status muffin_shard_spatial(muffin_plan P, const float *t, float *z, doub
   P->mu[0] = mu; P->gamma[0] = gamma;
   Group h = g;
   h.C = 1;
-  CK(launch_gradient(h.x, h.g, h.b, P->S, P->kspec, P->tw(), P->n, P->Lt, 1, P->ws, P->pp(),
+  CK(launch_gradient(h.x, h.g, h.b, P->S, P->kspec, P->tw(), P->twc(), P->n, P->Lt, 1, P->ws, P->pp(),
                      P->grad_chunk, P->fft_radix));
   WaveArgs w = P->wave(1);
   CK(wavelet_synthesis_prox(w, h, P->p.positivity, P->ws));
@@ -1731,7 +1733,7 @@ muffin_status muffin_op_gradient(muffin_plan P, const float *x, const float *dir
   }
   s = fetch(P, x, P->op_in, P->NL);
   if (s != MUFFIN_OK) return s;
-  CK(launch_gradient(P->op_in, P->op_out, bb, P->S, P->kspec, P->tw(), P->n, P->Lt, 1, P->ws,
+  CK(launch_gradient(P->op_in, P->op_out, bb, P->S, P->kspec, P->tw(), P->twc(), P->n, P->Lt, 1, P->ws,
                      nullptr, 0, P->fft_radix));
   s = store(P, P->op_out, g, P->NL);
   if (s != MUFFIN_OK) return s;

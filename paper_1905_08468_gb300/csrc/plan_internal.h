@@ -115,6 +115,9 @@ struct muffin_plan_s {
   // twiddle tables of the selected FFT plan
   const float2 *tw() const { return fft_radix == 8 && n >= 64 ? tw32 + tw_len16 : tw32; }
 
+  // twiddles of the gradient's column pass
+  const float2 *twc() const { return tw32 + tw_len16 + muffin::fft32_table_len(n, 8); }
+
   template <typename T>
   cudaError_t alloc(T **ptr, size_t count) {
     void *q = nullptr;
