@@ -299,7 +299,10 @@ cudaError_t launch_f32_t(const F32Args &a, cudaStream_t st, Prof *prof) {
 template <int L, int CH, int MODE>
 cudaError_t launch_f32(const F32Args &a, cudaStream_t st, Prof *prof) {
   const size_t tiles = (a.npix + FShape<L, 256>::PT - 1) / FShape<L, 256>::PT * a.B;
-  return tiles < 304 ? launch_f32_t<L, CH, MODE, 64>(a, st, prof)
+  // below a 256-thread CTA an SM the quarter-size tiles fill the chip better
+  // (64 x 64 x 32, three chains: 24.8 -> 18 us); from there on the wide tiles' longer
+  // rows win (256 x 256 x 32, three chains, 256 tiles: 43.7 against 35.1 us)
+  return tiles < 150 ? launch_f32_t<L, CH, MODE, 64>(a, st, prof)
                      : launch_f32_t<L, CH, MODE, 256>(a, st, prof);
 }
 
