@@ -271,8 +271,9 @@ typedef struct {
                                chain group; k > 0 = the three passes run k
                                images at a time, so the spectra stay in L2 */
   int32_t fft_radix;        /* largest radix of the gradient's FFT plan: 16
-                               (default) or 8 (n >= 64; 1024 = 8.8.8.2 instead
-                               of 16.16.4); results agree to FP32 rounding */
+                               (default) or 8 (from n = 128 on; 1024 = 8.8.8.2
+                               instead of 16.16.4; without effect on smaller
+                               images); results agree to FP32 rounding */
   int32_t group_order;      /* ADA-PT plans: 0 = one chain group's kernels
                                after the other's, 1 = both groups phase by
                                phase, 2 = the two groups concurrently on two

@@ -237,7 +237,7 @@ __device__ __forceinline__ const float2 *fft_middle(float2 *d, int pitch, int nt
   return tw;
 }
 
-// ---- in-place plan of the column pass (N >= 64): decimation in frequency with
+// ---- in-place plan of the column pass (N >= 32): decimation in frequency with
 // radices 16, 16 (N > 256) and a last one of 2 .. 16, backwards by the mirrored
 // stages, so that the last forward and the first inverse stage meet in registers
 // and no stage reorders.  Position p of a column then holds frequency
@@ -250,11 +250,11 @@ __host__ __device__ constexpr int cols_pos(int f, int N) {
 // twiddles exp(-2 pi i t k / len), k = 1 .. 15, at [(k - 1) len / 16 + t] for len = N
 // and (N > 256) len = N / 16
 __host__ __device__ constexpr int cols_table_len(int N) {
-  return N < 64 ? 1 : 15 * (N / 16) + (N > 256 ? 15 * (N / 256) : 0);
+  return N < 32 ? 1 : 15 * (N / 16) + (N > 256 ? 15 * (N / 256) : 0);
 }
 inline void cols_tables(int N, float2 *tab) {
   const double pi = 3.14159265358979323846;
-  if (N < 64) { tab[0] = make_float2(1.f, 0.f); return; }
+  if (N < 32) { tab[0] = make_float2(1.f, 0.f); return; }
   for (int len = N, off = 0; len == N || (N > 256 && len == N / 16); off += 15 * (len / 16), len /= 16)
     for (int k = 1; k < 16; ++k)
       for (int t = 0; t < len / 16; ++t) {

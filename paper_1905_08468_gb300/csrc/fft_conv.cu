@@ -11,8 +11,9 @@
 //               inverse FFT, in place;
 //   3. rows:    rebuild the Hermitian row spectra of two rows at a time,
 //               inverse FFT, subtract b, store.
-// The FP64 2D transform at the bottom is used only when a plan or call is
-// set up (PSF spectra, H^T y, H^T delta).
+// Images of 32 and 64 pixels a side go through the three in one kernel.
+// The 2D transforms at the bottom, in FP64 or on pairs of FP32 values, are used
+// only when a plan or call is set up (PSF spectra, H^T y, H^T delta).
 #include <cuda_runtime.h>
 
 #include "fft.cuh"
@@ -143,7 +144,7 @@ k_cols(float2 *__restrict__ S, const float *__restrict__ kspec, int L,
       Si[kThreads * u] = d[sb + ((kThreads * u) / n) * pitch + fpad((kThreads * u) % n)];
 }
 
-// The column pass from 64 rows on.  What bounds the Stockham form above is the
+// The column pass from 128 rows on.  What bounds the Stockham form above is the
 // shared-memory pipe (76 percent busy at 31 percent of the DRAM rate): an element
 // crosses it 16 times and the CTA meets at 16 barriers.  Here (in-place plan of
 // fft32.cuh) it crosses 8 times and meets at 4, columns come from and go to
@@ -322,6 +323,170 @@ k_rows_inv(const float2 *__restrict__ S, float *__restrict__ g_out,
       gi[2 * q * n + c] = v0;
       gi[(2 * q + 1) * n + c] = v1;
     }
+  }
+}
+
+// ---------------------------------------------------------------- small images
+// The whole gradient of an image of 32 or 64 pixels a side in one CTA: the half
+// spectra stay in shared memory between the passes, so an image is read and
+// written once and three launches become one.  A sequence belongs to N / 16 lanes
+// of a warp (16 values each, the in-place plan of fft32.cuh in two stages), so the
+// CTA meets only between the passes.  What bounds it: latency, at one image a CTA.
+// An iteration of a plain solve with one basis and one level, 1, 8 and 32 images:
+// 64 pixels 19.4 -> 17.6, 21.2 -> 19.7 and 22.7 -> 20.6 us; 32 pixels 19.4 -> 17.3,
+// 20.6 -> 19.5 and 23.6 -> 20.6; 768 images (three chains) 198 -> 190 and 97 -> 87.
+// At 128 pixels (141 KB, one CTA an SM) the three passes are faster: 22.6 against
+// 26.8 us with one image, 26.2 against 31.3 with 32, 529 against 549 with 768.
+template <int N>
+struct SmallGrad {
+  static constexpr int T = N / 16, RL = N / 16, GL = 16 / RL, nh = N / 2 + 1;
+  static constexpr int PITCH = N + N / 16 + 1;     // odd: 16 sequences, 16 bank pairs
+  static constexpr int NT = (nh * T + 31) / 32 * 32;
+  static constexpr size_t SMEM =
+      ((size_t)(N / 2 + nh) * PITCH + 15 * T) * sizeof(float2);
+};
+
+template <int N>
+__global__ void __launch_bounds__(SmallGrad<N>::NT)
+k_grad_small(const float *__restrict__ x, float *__restrict__ g_out, const float *__restrict__ bdata,
+             const float *__restrict__ kspec, int L, const float2 *__restrict__ twc) {
+  using G = SmallGrad<N>;
+  constexpr int T = G::T, nh = G::nh, half = N / 2;
+  extern __shared__ float2 sm2[];
+  float2 *rows = sm2, *cols = rows + half * G::PITCH, *tw = cols + nh * G::PITCH;
+  const int tid = threadIdx.x, s = tid / T, t = tid % T;
+  load_tw(tw, twc, 15 * T);
+  chain_enter();
+  const int img = blockIdx.x, band = img % L;
+  const size_t base = (size_t)img * N * N;
+  float2 v[16];
+  const bool row = s < half, col = s < nh;
+  float2 *dr = rows + (row ? s : 0) * G::PITCH, *dc = cols + (col ? s : 0) * G::PITCH;
+  const float *xr = x + base + (size_t)(2 * s) * N + t;
+  if (row)
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = make_float2(xr[r * T], xr[N + r * T]);
+  float kr[16];                                      // the column's multipliers
+  if (col) {
+    const float *K = kspec + ((size_t)band * nh + s) * N;
+#pragma unroll
+    for (int g = 0; g < G::GL; ++g)
+#pragma unroll
+      for (int e = 0; e < G::RL; ++e) kr[g * G::RL + e] = __ldg(K + (t + g * T) * G::RL + e);
+  }
+  __syncthreads();                                   // the table
+  // every lane meets the warp barriers, with a sequence or without
+  if (row) {
+    dft16<false>(v);
+    dr[fpad(t)] = v[0];
+#pragma unroll
+    for (int r = 1; r < 16; ++r) dr[fpad(r * T + t)] = cmul(v[out_slot<16>(r)], tw[(r - 1) * T + t]);
+  }
+  __syncwarp();
+  if (row) {
+#pragma unroll
+    for (int g = 0; g < G::GL; ++g) {
+      float2 u[G::RL];
+#pragma unroll
+      for (int e = 0; e < G::RL; ++e) u[e] = dr[fpad((t + g * T) * G::RL + e)];
+      dftR<G::RL, false>(u);
+#pragma unroll
+      for (int e = 0; e < G::RL; ++e) dr[fpad((t + g * T) * G::RL + e)] = u[out_slot<G::RL>(e)];
+    }
+  }
+  __syncthreads();
+  // half spectra of the two rows of a pair (see k_rows_fwd)
+  for (int i = tid; i < nh * half; i += G::NT) {
+    const int k = i / half, q = i % half;
+    const float2 *d = rows + q * G::PITCH;
+    const float2 Z = d[fpad(cols_pos(k, N))], Zc = d[fpad(cols_pos((N - k) & (N - 1), N))];
+    float2 *o = cols + k * G::PITCH;
+    o[fpad(2 * q)] = make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y - Zc.y));
+    o[fpad(2 * q + 1)] = make_float2(0.5f * (Z.y + Zc.y), 0.5f * (Zc.x - Z.x));
+  }
+  __syncthreads();
+  // columns: forward, multiply, inverse, in place
+  {
+    if (col)
+#pragma unroll
+      for (int r = 0; r < 16; ++r) v[r] = dc[fpad(t + r * T)];
+    __syncwarp();
+    if (col) {
+      dft16<false>(v);
+      dc[fpad(t)] = v[0];
+#pragma unroll
+      for (int r = 1; r < 16; ++r) dc[fpad(r * T + t)] = cmul(v[out_slot<16>(r)], tw[(r - 1) * T + t]);
+    }
+    __syncwarp();
+    if (col) {
+#pragma unroll
+      for (int g = 0; g < G::GL; ++g) {
+        float2 u[G::RL], z[G::RL];
+#pragma unroll
+        for (int e = 0; e < G::RL; ++e) u[e] = dc[fpad((t + g * T) * G::RL + e)];
+        dftR<G::RL, false>(u);
+#pragma unroll
+        for (int e = 0; e < G::RL; ++e) {
+          const float2 y = u[out_slot<G::RL>(e)];
+          z[e] = make_float2(y.x * kr[g * G::RL + e], y.y * kr[g * G::RL + e]);
+        }
+        dftR<G::RL, true>(z);
+#pragma unroll
+        for (int e = 0; e < G::RL; ++e) dc[fpad((t + g * T) * G::RL + e)] = z[out_slot<G::RL>(e)];
+      }
+    }
+    __syncwarp();
+    if (col) {
+      v[0] = dc[fpad(t)];
+#pragma unroll
+      for (int r = 1; r < 16; ++r) v[r] = cmulc(dc[fpad(r * T + t)], tw[(r - 1) * T + t]);
+      dft16<true>(v);
+    }
+    __syncwarp();
+    if (col)
+#pragma unroll
+      for (int r = 0; r < 16; ++r) dc[fpad(t + r * T)] = v[out_slot<16>(r)];
+  }
+  __syncthreads();
+  // Hermitian row spectra of the pairs (see k_rows_inv)
+  for (int i = tid; i < nh * half; i += G::NT) {
+    const int k = i / half, q = i % half;
+    float2 A = cols[k * G::PITCH + fpad(2 * q)], B = cols[k * G::PITCH + fpad(2 * q + 1)];
+    if (k == 0 || k == half) { A.y = 0.f; B.y = 0.f; }
+    float2 *d = rows + q * G::PITCH;
+    d[fpad(cols_pos(k, N))] = make_float2(A.x - B.y, A.y + B.x);                       // A + i B
+    if (k > 0 && k < half)
+      d[fpad(cols_pos(N - k, N))] = make_float2(A.x + B.y, B.x - A.y);   // conj A + i conj B
+  }
+  __syncthreads();
+  if (row) {
+#pragma unroll
+    for (int g = 0; g < G::GL; ++g) {
+      float2 u[G::RL];
+#pragma unroll
+      for (int e = 0; e < G::RL; ++e) u[e] = dr[fpad((t + g * T) * G::RL + e)];
+      dftR<G::RL, true>(u);
+#pragma unroll
+      for (int e = 0; e < G::RL; ++e) dr[fpad((t + g * T) * G::RL + e)] = u[out_slot<G::RL>(e)];
+    }
+  }
+  __syncwarp();
+  if (!row) return;
+  v[0] = dr[fpad(t)];
+#pragma unroll
+  for (int r = 1; r < 16; ++r) v[r] = cmulc(dr[fpad(r * T + t)], tw[(r - 1) * T + t]);
+  dft16<true>(v);
+  float *gr = g_out + base + (size_t)(2 * s) * N + t;
+  const float *br = bdata && img < L ? bdata + base + (size_t)(2 * s) * N + t : nullptr;
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    float2 z = v[out_slot<16>(r)];
+    if (br) {
+      z.x -= __ldg(br + r * T);
+      z.y -= __ldg(br + N + r * T);
+    }
+    gr[r * T] = z.x;
+    gr[N + r * T] = z.y;
   }
 }
 
@@ -526,7 +691,7 @@ __global__ void k_make_kspec(const double2 *__restrict__ hh, float *__restrict__
   for (int ky = threadIdx.x; ky < n; ky += blockDim.x) {
     const double v = h[ky].x * h[ky].x + h[ky].y * h[ky].y;
     m = max(m, (unsigned long long)__double_as_longlong(fabs(v)));
-    k[n < 64 ? ky : cols_pos(ky, n)] = (float)(v * scale);
+    k[n < 32 ? ky : cols_pos(ky, n)] = (float)(v * scale);
   }
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
@@ -552,51 +717,57 @@ cudaError_t gradient_n(const float *x, float *g, const float *b, float2 *S,
                        cudaStream_t st, Prof *prof, int chunk) {
   constexpr int n = NN;
   const int ntot = C * L;
-  const int RB = 2 * row_pairs(n);                  // real rows per CTA (even)
-  const int CB = seqs_per_cta(n);                   // columns per CTA
   const int nh = (n >> 1) + 1;
-  const int pitch = n + (n >> 4);
-  const int tlen = fft_table_len(n, RMAX);
-  const size_t smr = ((size_t)(RB / 2) * row_pitch(n) + tlen) * sizeof(float2);
-  const size_t smc = ((size_t)CB * pitch + (n >= 64 ? cols_table_len(n) : tlen)) * sizeof(float2);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_rows_fwd<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_rows_inv<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if constexpr (NN >= 64)
-      cudaFuncSetAttribute(k_cols_dif<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    else
-      cudaFuncSetAttribute(k_cols<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr = true;
-  }
   const double img = (double)n * n, spec = (double)nh * n * 8.0;
   const double fft = 5.0 * n * ilog2(n);   // flops of one length-n complex FFT
-  const int step = chunk > 0 && chunk < ntot ? chunk : ntot;
   // the whole call: x read, g written, b read, |h_hat|^2 read once per
-  // band, the spectra of every image written and read twice
+  // band, and in three passes the spectra of every image written and read twice
   ProfScope all(prof, "grad_total",
-                ntot * (img * 8.0 + 4.0 * spec) + (b ? (double)L * img * 4.0 : 0.0) +
+                ntot * (img * 8.0 + (n < 32 || n > 64 ? 4.0 * spec : 0.0)) + (b ? (double)L * img * 4.0 : 0.0) +
                     (double)L * nh * n * 4.0,
                 ntot * (double)(n + 2 * nh) * fft, st);
-  for (int i0 = 0; i0 < ntot; i0 += step) {
-    const int nimg = step < ntot - i0 ? step : ntot - i0;
-    const int nb = b ? (i0 < L ? (L - i0 < nimg ? L - i0 : nimg) : 0) : 0;   // images with b
-    {
-      ProfScope ps(prof, "grad_rows_fwd", nimg * (img * 4.0 + spec),
-                   nimg * (n / 2.0) * fft, st);
-      launch_chain(k_rows_fwd<NN, RMAX>, dim3(n / RB, nimg), kThreads, smr, st, x, S, tw, tlen, i0);
+  if constexpr (NN == 32 || NN == 64) {
+    using G = SmallGrad<NN>;
+    cudaFuncSetAttribute(k_grad_small<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    launch_chain(k_grad_small<NN>, dim3(ntot), G::NT, G::SMEM, st, x, g, b, kspec, L, twc);
+  } else {
+    const int RB = 2 * row_pairs(n);                  // real rows per CTA (even)
+    const int CB = seqs_per_cta(n);                   // columns per CTA
+    const int pitch = n + (n >> 4);
+    const int tlen = fft_table_len(n, RMAX);
+    const size_t smr = ((size_t)(RB / 2) * row_pitch(n) + tlen) * sizeof(float2);
+    const size_t smc = ((size_t)CB * pitch + (n >= 128 ? cols_table_len(n) : tlen)) * sizeof(float2);
+    static bool attr = false;
+    if (!attr) {
+      cudaFuncSetAttribute(k_rows_fwd<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      cudaFuncSetAttribute(k_rows_inv<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      if constexpr (NN >= 128)
+        cudaFuncSetAttribute(k_cols_dif<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      else
+        cudaFuncSetAttribute(k_cols<NN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      attr = true;
     }
-    {
-      ProfScope ps(prof, "grad_cols", nimg * 2.0 * spec + (double)nimg * nh * n * 4.0,
-                   nimg * (double)nh * 2.0 * fft, st);
-      const dim3 grid((nh + CB - 1) / CB, nimg);
-      if constexpr (NN >= 64) launch_chain(k_cols_dif<NN>, grid, kThreads, smc, st, S, kspec, L, twc, i0);
-      else launch_chain(k_cols<NN, RMAX>, grid, kThreads, smc, st, S, kspec, L, tw, tlen, i0);
-    }
-    {
-      ProfScope ps(prof, "grad_rows_inv", nimg * (spec + img * 4.0) + nb * img * 4.0,
-                   nimg * (n / 2.0) * fft, st);
-      launch_chain(k_rows_inv<NN, RMAX>, dim3(n / RB, nimg), kThreads, smr, st, S, g, b, L, tw, tlen, i0);
+    const int step = chunk > 0 && chunk < ntot ? chunk : ntot;
+    for (int i0 = 0; i0 < ntot; i0 += step) {
+      const int nimg = step < ntot - i0 ? step : ntot - i0;
+      const int nb = b ? (i0 < L ? (L - i0 < nimg ? L - i0 : nimg) : 0) : 0;   // images with b
+      {
+        ProfScope ps(prof, "grad_rows_fwd", nimg * (img * 4.0 + spec),
+                     nimg * (n / 2.0) * fft, st);
+        launch_chain(k_rows_fwd<NN, RMAX>, dim3(n / RB, nimg), kThreads, smr, st, x, S, tw, tlen, i0);
+      }
+      {
+        ProfScope ps(prof, "grad_cols", nimg * 2.0 * spec + (double)nimg * nh * n * 4.0,
+                     nimg * (double)nh * 2.0 * fft, st);
+        const dim3 grid((nh + CB - 1) / CB, nimg);
+        if constexpr (NN >= 128) launch_chain(k_cols_dif<NN>, grid, kThreads, smc, st, S, kspec, L, twc, i0);
+        else launch_chain(k_cols<NN, RMAX>, grid, kThreads, smc, st, S, kspec, L, tw, tlen, i0);
+      }
+      {
+        ProfScope ps(prof, "grad_rows_inv", nimg * (spec + img * 4.0) + nb * img * 4.0,
+                     nimg * (n / 2.0) * fft, st);
+        launch_chain(k_rows_inv<NN, RMAX>, dim3(n / RB, nimg), kThreads, smr, st, S, g, b, L, tw, tlen, i0);
+      }
     }
   }
   return cudaGetLastError();

@@ -95,7 +95,7 @@ int set_last_error_code(int s, const char *msg);
 // chunk > 0: the three passes run over `chunk` images at a time (S then
 // needs room for chunk images only and stays in L2 between the passes);
 // chunk <= 0: each pass over all images at once.
-// radix 16 (default) or 8 (n >= 64): the largest radix of the FFT plan; tw
+// radix 16 (default) or 8 (n >= 128): the largest radix of the row passes; tw
 // must hold that plan's twiddle tables (fft32_tables with the same radix).
 cudaError_t launch_gradient(const float *x, float *g, const float *b,
                             float2 *S, const float *kspec, const float2 *tw, const float2 *twc,
@@ -106,7 +106,7 @@ cudaError_t launch_gradient(const float *x, float *g, const float *b,
 // the plan whose largest radix is `radix`.
 int fft32_table_len(int n, int radix = 16);
 void fft32_tables(int n, float2 *tab, int radix = 16);
-// Twiddles of the column pass from 64 rows on (twc above; any radix).
+// Twiddles of the column pass from 32 rows on (twc above; any radix).
 int fft32_cols_table_len(int n);
 void fft32_cols_tables(int n, float2 *tab);
 
@@ -135,7 +135,7 @@ cudaError_t convolve_real(const float *x, const ImageStat *stat, const double2 *
 cudaError_t c64_real_to_f32(const double2 *in, float *out, double scale,
                             size_t count, cudaStream_t st);
 // kspec[l][kx][.] = |hh[l][kx][ky]|^2 * scale for kx < n/2+1, in the column pass's
-// order of ky (cols_pos in fft32.cuh; natural below 64 rows); hmax[l] = the
+// order of ky (cols_pos in fft32.cuh; natural below 32 rows); hmax[l] = the
 // largest |hh[l]|^2 (NaN if any is)
 cudaError_t make_kspec(const double2 *hh, float *kspec, double scale, int n,
                        int L, double *hmax, cudaStream_t st);
