@@ -15,13 +15,23 @@
 // warp and band), splits its row of the A operand into TF32 halves itself,
 // and reads its accumulator row straight from tensor memory (the warp's lane
 // quadrant), so no shared-memory staging of v or t is needed.  The raw x~
-// and x tiles of a chain arrive by 16-byte cp.async into the A buffers
-// (free before the split), so the whole 64 KB is in flight at once.
+// and x tiles of a chain arrive by 16-byte cp.async into the A buffers, requested
+// as soon as the chain before has been through its second product, so the whole
+// 64 KB is in flight while that chain's t is written.
 //
 // A CTA runs two independent groups of 8 warps that share the C tables but
 // own their A tiles, tensor-memory columns (128, or 256 with three chains,
 // where the d/dgamma chain accumulates onto chain 0's products) and
-// mbarrier, so one group's global traffic overlaps the other's MMAs.  Waits on the mbarriers are
+// mbarrier, so one group's global traffic overlaps the other's MMAs.  What bounds
+// it: the chain of load, split, product, dual update, product, store in a group.
+// Requested at the top of a chain, with an L2 prefetch of the next, and with
+// neighbouring tiles on a CTA's groups, the loads left 1024 x 1024, three chains at
+// 915 us; now 789 (5.1 TB/s).  Few tiles, an iteration of a plain solve: 32 x 32 34.3
+// -> 25.8 us, 64 x 64 34.2 -> 26.0, 256 x 256 102 -> 93 (a CTA a tile, 16-byte table
+// loads before the wait for the kernel in front); ADA-PT 64 x 64 143 -> 105.  The
+// old duals requested before the loads as well, with the prefetch and neighbouring
+// tiles: 761 us there, but 98 us at 256 x 256, one chain, and 508 against 501 with
+// three.  Waits on the mbarriers are
 // bounded: on time-out the kernel raises an error flag, waits once more and
 // frees its tensor memory; the host turns the flag into MUFFIN_ETIMEOUT.  A
 // host-side test hook makes the kernel skip its products so that this path
@@ -115,20 +125,6 @@ __device__ __forceinline__ void stage_raw(const float *xt, const float *x, size_
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// the band rows stage_raw will read for (base, p0), into L2 ahead of time:
-// one bulk prefetch per (band, array), 16-byte aligned (p0 is a multiple of
-// the 128-pixel tile) and cut at the end of the pixel range
-__device__ __forceinline__ void prefetch_raw(const float *xt, const float *x, size_t base,
-                                             size_t N, size_t p0, int gt) {
-  if (gt >= 2 * TL || p0 >= N) return;
-  const size_t cnt = (N - p0 < (size_t)TM ? N - p0 : (size_t)TM) & ~(size_t)3;
-  if (cnt == 0) return;
-  const int l = gt >> 1;
-  const float *src = (gt & 1 ? x : xt) + base + (size_t)l * N + p0;
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)(cnt * 4))
-               : "memory");
-}
-
 __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(GT) : "memory");
 }
@@ -204,7 +200,6 @@ __device__ __forceinline__ void store_split(uint8_t *ahi, uint8_t *alo, int row,
 
 template <int CH>
 __global__ void __launch_bounds__(CTA_T, 1) k_dct_tc(TcArgs a) {
-  chain_enter();
   extern __shared__ uint8_t raw[];
   __shared__ __align__(8) uint64_t mbar[NG];
   __shared__ uint32_t tmem_base;
@@ -217,8 +212,9 @@ __global__ void __launch_bounds__(CTA_T, 1) k_dct_tc(TcArgs a) {
   const float *src[4] = {a.chi, a.clo, a.cthi, a.ctlo};
 #pragma unroll
   for (int m = 0; m < 4; ++m)
-    for (int i = tid; i < TL * TL; i += CTA_T)
-      *reinterpret_cast<float *>(cth[m] + cm_off(i / TL, i % TL)) = src[m][i];
+    for (int i = 4 * tid; i < TL * TL; i += 4 * CTA_T)
+      *reinterpret_cast<float4 *>(cth[m] + cm_off(i / TL, i % TL)) =
+          __ldg(reinterpret_cast<const float4 *>(src[m] + i));
   if (tid < NG) {
     const uint32_t mb = (uint32_t)__cvta_generic_to_shared(&mbar[tid]);
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory");
@@ -234,6 +230,8 @@ __global__ void __launch_bounds__(CTA_T, 1) k_dct_tc(TcArgs a) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+
+  chain_enter();           // the tables are the plan's, the rest is the iteration's
 
   const uint32_t mb = (uint32_t)__cvta_generic_to_shared(&mbar[g]);
   const uint32_t quad = (uint32_t)(wg & 3), h = (uint32_t)(wg >> 2);
@@ -258,8 +256,17 @@ __global__ void __launch_bounds__(CTA_T, 1) k_dct_tc(TcArgs a) {
   const int row = (int)quad * 32 + lane;          // pixel within the tile = accumulator lane
   uint32_t ph = 0;
   bool ok = true;
+  // the raw tiles of chain c of a tile, through the A buffers
+  const auto stage = [&](int tile, int c) {
+    const int cube = tile / tpc;
+    stage_raw(a.xt + c * CS, a.x + c * CS, (size_t)cube * TL * N, N,
+              (size_t)(tile - cube * tpc) * TM, gt, ahi, alo);
+  };
 
-  for (int tile = blockIdx.x * NG + g; tile < ntiles && ok; tile += gridDim.x * NG) {
+  // a CTA's groups take tiles a grid apart, so that few tiles get a CTA each
+  const int first = blockIdx.x + g * gridDim.x, step = gridDim.x * NG;
+  if (first < ntiles) stage(first, 0);
+  for (int tile = first; tile < ntiles && ok; tile += step) {
     const int cube = tile / tpc;
     const size_t p = (size_t)(tile - cube * tpc) * TM + row;
     const bool valid = p < N;
@@ -272,21 +279,8 @@ __global__ void __launch_bounds__(CTA_T, 1) k_dct_tc(TcArgs a) {
       const bool mix = CH == 3 && c == 2;          // accumulate onto chain 0's products
       const uint32_t off1 = (CH == 3 && c == 1) ? 128u : 0u, off2 = off1 + 64u;
       // ---- first product: z = 2x~ - x (gamma z' for d/dgamma, whose + z is
-      // chain 0's product already in tensor memory); the raw tiles are staged
-      // through the A buffers, free at this point
-      const size_t tile_base = (size_t)cube * TL * N;
-      const size_t p0 = p - row;
+      // chain 0's product already in tensor memory)
       float z[32];
-      stage_raw(a.xt + c * CS, a.x + c * CS, tile_base, N, p0, gt, ahi, alo);
-      {   // the next (tile, chain) of this group, into L2 while this one runs
-        const int nt = c + 1 < CH ? tile : tile + (int)gridDim.x * NG;
-        const int nc = c + 1 < CH ? c + 1 : 0;
-        if (nt < ntiles) {
-          const int ncube = nt / tpc;
-          prefetch_raw(a.xt + nc * CS, a.x + nc * CS, (size_t)ncube * TL * N, N,
-                       (size_t)(nt - ncube * tpc) * TM, gt);
-        }
-      }
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       group_sync(g);
 #pragma unroll
@@ -355,6 +349,9 @@ __global__ void __launch_bounds__(CTA_T, 1) k_dct_tc(TcArgs a) {
       group_sync(g);
       if (bail[g]) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // the A buffers are free: the next (tile, chain) while this one is written
+      if (c + 1 < CH) stage(tile, c + 1);
+      else if (tile + step < ntiles) stage(tile + step, 0);
       tmem_row32(lanes + off2 + 32u * h, acc);
       const float s2 = (c == 2) ? al : gamma * al;
       if (valid) {
@@ -389,8 +386,7 @@ cudaError_t launch_tc(const TcArgs &a, cudaStream_t st, Prof *prof) {
   }
   const size_t N = a.npix;
   const size_t ntiles = ((N + TM - 1) / TM) * (size_t)a.B;
-  const size_t ctas = (ntiles + NG - 1) / NG;
-  const size_t grid = ctas < (size_t)sms ? ctas : (size_t)sms;
+  const size_t grid = ntiles < (size_t)sms ? ntiles : (size_t)sms;
   const double vox = (double)N * TL * a.B;
   ProfScope ps(prof, "spectral_dual", CH * vox * 20.0, 2.0 * CH * 2.0 * TL * vox, st);
   launch_chain(k_dct_tc<CH>, (unsigned)grid, CTA_T, SMEM, st, a);

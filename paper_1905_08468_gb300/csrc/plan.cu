@@ -140,7 +140,7 @@ muffin_status validate(const muffin_params *p) {
 // O(log L) work per voxel and is bound by its memory traffic, while a dense
 // product grows with L (1024 x 1024 x 256, one chain: 1.1 ms against 7.0 ms in
 // 3xTF32) and keeps more error.  At 64 bands the tcgen05 kernel is the faster one
-// with three chains at 1024 x 1024 (0.94 against 1.00 ms) and stays.
+// with three chains at 1024 x 1024 (0.79 against 1.00 ms) and stays.
 bool spectral_f32(const muffin_params *p) {
   const int L = p->nbands;
   return p->precision == 1 || (L >= 2 && L <= 1024 && L != 64 && (L & (L - 1)) == 0);
