@@ -44,7 +44,7 @@ CROP = dict(n=128, L=64, iters=2)
 # ncu capture (profiles/), valid only while the kernel's source file is the
 # one the counters were taken on (sha256 prefix).
 CAPTURED_TRAFFIC = {
-    "ana_level1_dual": ("paper_1905_08468_gb300/csrc/wavelet.cu", "d2db0c7118e4171c", 61.63),
+    "ana_level1_dual": ("paper_1905_08468_gb300/csrc/ana_cols.cu", "1fc595bba2f9021e", 62.92),
 }
 
 
@@ -249,9 +249,10 @@ def workload_config(args, oracle=False) -> dict:
            "window": args.window,
            "wavelets": ("IUWT (starlet), 3 scales" if getattr(args, "dictionary", "daubechies") == "iuwt"
                         else "db1..db8, 3 levels"),
-           "spectral": ("DCT-II in FP32 on the CUDA cores (fast DCT, one complex DFT per pixel pair)"
-                        if getattr(args, "precision", "tf32") == "fp32" else
-                        "DCT-II, 3xTF32 products on the tensor cores (tcgen05 for 64 bands, else mma.sync)"),
+           "spectral": ("DCT-II, 3xTF32 products on the tensor cores (tcgen05)"
+                        if L == 64 and getattr(args, "precision", "tf32") != "fp32" else
+                        "DCT-II in FP32 on the CUDA cores (fast DCT, one complex DFT per pixel pair)"
+                        if L & (L - 1) == 0 else "DCT-II in FP32 on the CUDA cores (dense, folded)"),
            "chains": 1 if plain else 6,
            "theta0": None if plain else list(THETA0), "eta": None if plain else list(ETA),
            "l2": "inputs larger than L2 (state ~26 GB per cube at 1024^2 x 64 ADA-PT)"}
@@ -498,8 +499,8 @@ def main() -> None:
     ap.add_argument("--schedule", default="",
                     help="schedule overrides after tuning, e.g. ana_pipe=0,group_order=1")
     ap.add_argument("--precision", default="tf32", choices=["tf32", "fp32"],
-                    help="spectral DCT: 3xTF32 tensor-core products (default) or the FP32 "
-                         "fast DCT on the CUDA cores")
+                    help="spectral DCT: the default kernel of the band count (64 bands: 3xTF32 "
+                         "tensor-core products) or the FP32 fast DCT on the CUDA cores")
     ap.add_argument("--grad-chunk", type=int, default=-1,
                     help="images per pass of the gradient FFTs (-1: the tuner's choice)")
     ap.add_argument("--no-cufft", action="store_true",

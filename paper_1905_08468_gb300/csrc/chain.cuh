@@ -3,8 +3,8 @@
 // CTAs are placed as soon as that one's have left; chain_enter(), the first
 // thing a kernel of the chain does with memory that another one writes, waits
 // until the kernel before has finished and its results are visible.  This takes
-// part of the launch latency out of every boundary: 64 x 64 x 8 (11 kernels an
-// iteration, 9 since the gradient is one) 43.5 -> 39 us an iteration, 256 x 256 x 37 1-2 percent, large cubes
+// part of the launch latency out of every boundary: 64 x 64 x 8 (10 kernels an
+// iteration, 8 since the gradient is one) 43.5 -> 39 us an iteration, 256 x 256 x 37 1-2 percent, large cubes
 // unchanged.  No kernel triggers its dependents early: waiting CTAs then hold
 // registers and shared memory beside the running kernel's last waves (1024 x
 // 1024 x 256: 196 -> 210 ms a pass, triggered before or after the wait).

@@ -23,7 +23,7 @@
 // own their A tiles, tensor-memory columns (128, or 256 with three chains,
 // where the d/dgamma chain accumulates onto chain 0's products) and
 // mbarrier, so one group's global traffic overlaps the other's MMAs.  What bounds
-// it: the chain of load, split, product, dual update, product, store in a group.
+// it: the order of load, split, product, dual update, product and store in a group.
 // Requested at the top of a chain, with an L2 prefetch of the next, and with
 // neighbouring tiles on a CTA's groups, the loads left 1024 x 1024, three chains at
 // 915 us; now 789 (5.1 TB/s).  Few tiles, an iteration of a plain solve: 32 x 32 34.3
