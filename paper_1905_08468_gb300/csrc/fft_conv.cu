@@ -728,7 +728,7 @@ cudaError_t gradient_n(const float *x, float *g, const float *b, float2 *S,
                 ntot * (double)(n + 2 * nh) * fft, st);
   if constexpr (NN == 32 || NN == 64) {
     using G = SmallGrad<NN>;
-    cudaFuncSetAttribute(k_grad_small<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    static_assert(G::SMEM <= 48 * 1024, "no opt-in needed");
     launch_chain(k_grad_small<NN>, dim3(ntot), G::NT, G::SMEM, st, x, g, b, kspec, L, twc);
   } else {
     const int RB = 2 * row_pairs(n);                  // real rows per CTA (even)
@@ -779,7 +779,7 @@ cudaError_t launch_gradient(const float *x, float *g, const float *b,
                             float2 *S, const float *kspec, const float2 *tw, const float2 *twc,
                             int n, int L, int C, cudaStream_t st, Prof *prof, int chunk,
                             int radix) {
-  const bool r8 = radix == 8 && n >= 64;   // the alternative plan exists from n = 64
+  const bool r8 = radix == 8;              // the alternative plan exists from n = 128
 #define MUFFIN_GRAD(NN)                                                                    \
   return r8 ? gradient_n<NN, 8>(x, g, b, S, kspec, tw, twc, L, C, st, prof, chunk)              \
             : gradient_n<NN, 16>(x, g, b, S, kspec, tw, twc, L, C, st, prof, chunk)
@@ -790,7 +790,7 @@ cudaError_t launch_gradient(const float *x, float *g, const float *b,
     case 8: MUFFIN_GRAD16(8);
     case 16: MUFFIN_GRAD16(16);
     case 32: MUFFIN_GRAD16(32);
-    case 64: MUFFIN_GRAD(64);
+    case 64: MUFFIN_GRAD16(64);
     case 128: MUFFIN_GRAD(128);
     case 256: MUFFIN_GRAD(256);
     case 512: MUFFIN_GRAD(512);
