@@ -34,7 +34,7 @@ struct ImageStat {
   unsigned max_bits;    // bits of the largest |x| among the finite values
   unsigned nonfinite;   // NaN/Inf entries
   unsigned negative;    // entries < 0
-  unsigned pad;
+  unsigned infinite;    // the nonfinite ones that are Inf
 };
 
 // The power of two that takes a spectrum with largest |h|^2 = m2 to a largest

@@ -533,7 +533,8 @@ __global__ void k_transpose64(const double2 *__restrict__ in,
 // An image is scaled by a power of two (exact) to a largest magnitude in
 // [1, 2), and a band's spectrum h by one to [1, 2) or [2, 4), so that a faint
 // band keeps its own precision beside a bright one; a band with NaN/Inf enters
-// as zero and comes out as NaN, and leaves its neighbour alone.  Spectra stay
+// as zero and comes out as NaN (a PSF with Inf and no NaN as an infinite spectrum,
+// which no step size admits), and leaves its neighbour alone.  Spectra stay
 // transposed ([kx][ky]): one transpose each way.
 
 // 2^-e of an image from its statistics: 1 for a zero image, NaN if any value is
@@ -549,6 +550,10 @@ struct Pairs {
   const double *hmax;           // [images] largest |h|^2 (not finite: h is not)
   __device__ double scale(int img) const { return image_scale(stat[img]); }
   __device__ double hscale(int img) const { return spectrum_scale(hmax[img]); }
+  // Inf entries and no NaN: the spectrum is infinite (beside a NaN it is NaN)
+  __device__ bool infinite(int img) const {
+    return stat[img].infinite && stat[img].infinite == stat[img].nonfinite;
+  }
   __device__ int first(int p) const { return p / per_cube * L + 2 * (p % per_cube); }
   __device__ bool second(int p) const { return 2 * (p % per_cube) + 1 < L; }
 };
@@ -632,12 +637,14 @@ __global__ void k_pair_unpack(const double2 *__restrict__ z, double2 *__restrict
   const double2 *zr = z + p * N + row, *zm = z + p * N + (size_t)((n - kx) & (n - 1)) * n;
   const bool two = P.second(p);
   const double ra = 1.0 / P.scale(ia), rb = two ? 1.0 / P.scale(ia + 1) : 0.0;
+  const bool infa = P.infinite(ia), infb = two && P.infinite(ia + 1);
+  const double2 inf = make_double2(HUGE_VAL, 0.0);
   double2 *ha = hh + ia * N + row, *hb = ha + N;
   for (int ky = threadIdx.x; ky < n; ky += blockDim.x) {
     double2 A, B;
     pair_split(zr[ky], zm[(n - ky) & (n - 1)], A, B);
-    ha[ky] = make_double2(ra * A.x, ra * A.y);
-    if (two) hb[ky] = make_double2(rb * B.x, rb * B.y);
+    ha[ky] = infa ? inf : make_double2(ra * A.x, ra * A.y);
+    if (two) hb[ky] = infb ? inf : make_double2(rb * B.x, rb * B.y);
   }
 }
 

@@ -73,11 +73,15 @@ __global__ void k_image_stats(const float *__restrict__ x, size_t N, ImageStat *
   const size_t step = (size_t)gridDim.x * blockDim.x;
   size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   float m = 0.f;
-  unsigned bad = 0, neg = 0;
+  unsigned bad = 0, neg = 0, inf = 0;
   auto one = [&](float v) {
     const float a = fabsf(v);
-    if (isfinite(v)) m = fmaxf(m, a);
-    else ++bad;
+    if (isfinite(v)) {
+      m = fmaxf(m, a);
+    } else {
+      ++bad;
+      inf += isinf(v) ? 1u : 0u;
+    }
     neg += v < 0.f;
   };
   if ((N & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
@@ -94,12 +98,14 @@ __global__ void k_image_stats(const float *__restrict__ x, size_t N, ImageStat *
     m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     bad += __shfl_xor_sync(0xffffffffu, bad, o);
     neg += __shfl_xor_sync(0xffffffffu, neg, o);
+    inf += __shfl_xor_sync(0xffffffffu, inf, o);
   }
   if ((threadIdx.x & 31) == 0) {
     ImageStat *s = stat + blockIdx.y;
     if (m > 0.f) atomicMax(&s->max_bits, __float_as_uint(m));
     if (bad) atomicAdd(&s->nonfinite, bad);
     if (neg) atomicAdd(&s->negative, neg);
+    if (inf) atomicAdd(&s->infinite, inf);
   }
 }
 

@@ -193,8 +193,9 @@ muffin_status adjoint(muffin_plan P, const float *y_dev, int c0, int nimg, doubl
   return MUFFIN_OK;
 }
 
-// beta = the largest |h_hat|^2 of the cubes [c0, c1), from make_kspec (a band that
-// is not a number is passed over here; it shows in the results)
+// beta = the largest |h_hat|^2 of the cubes [c0, c1), from make_kspec; refused where
+// it is zero or infinite.  A band that is not a number is passed over: its gradient
+// is NaN, and the projection onto the positive orthant makes zeros of it.
 muffin_status read_lipschitz(muffin_plan P, int c0, int c1, const char *what) {
   std::vector<double> m((size_t)(c1 - c0) * P->L);
   CK(cudaMemcpyAsync(m.data(), P->hmax + (size_t)c0 * P->L, m.size() * sizeof(double),
