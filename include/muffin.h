@@ -223,12 +223,13 @@ typedef struct {
 /* Times each candidate configuration on this plan's own buffers (a few
  * iterations of every chain group it advances: two groups of three chains
  * with sure = 1, one plain group otherwise), keeps the fastest and caches it
- * per shape (n, bands, batch, chains, levels, bases, spectral precision, SM
- * count, device name): in process, and in the text file `cache_path` when it
+ * per shape (n, bands, batch, chains, levels, bases, spectral precision, the
+ * kernels it was timed on, SM count, device name): in process, and in the text file `cache_path` when it
  * is not NULL (read first, one line "muffin-tune-6 <key> <syn_packed>
  * <dct_ctas> <tcgen05> <grad_chunk> <fft_radix> <group_order> <ana_ring>
  * <ana_pipe>"
- * appended per new shape; lines that do not parse are ignored).  The timing iterations overwrite the plan's iterate state: a
+ * appended per new shape; lines that do not parse, or that were timed on kernels whose
+ * choices meant something else, are ignored).  The timing iterations overwrite the plan's iterate state: a
  * following solve or sure_tune must start cold (warm = 0; a warm call
  * returns MUFFIN_ESTATE), and captured graphs are rebuilt.  info may be NULL.
  * Errors: EINVAL (plan NULL), ECUDA. */

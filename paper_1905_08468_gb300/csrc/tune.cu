@@ -30,6 +30,11 @@ struct Choice {
   int ana_pipe = 0;    // analysis tiles of the other height than the rule's
 };
 
+// The kernels that a stored choice was timed on, part of its key: to be raised
+// when a choice comes to mean another launch.  1 (lines without the field): dct_ctas
+// and dct_tc = 0 on mma.sync, ana_pipe the chain-major level-1 analysis.
+constexpr int kKernels = 2;
+
 std::mutex g_mu;
 std::map<std::string, Choice> g_cache;
 
@@ -44,9 +49,9 @@ std::string shape_key(muffin_plan P) {
     if (ch == ' ' || ch == '\t') ch = '_';
   char buf[256];
   std::snprintf(buf, sizeof buf,
-                "n=%d,L=%d,B=%d,C=%d,J=%d,K=%d,dict=%d,sure=%d,prec=%d,sm=%d,dev=%s", P->n,
+                "n=%d,L=%d,B=%d,C=%d,J=%d,K=%d,dict=%d,sure=%d,prec=%d,kernels=%d,sm=%d,dev=%s", P->n,
                 P->L, P->B, P->Cmax, P->J, P->K, P->dict, P->p.sure ? 1 : 0, P->p.precision,
-                sms, name.c_str());
+                kKernels, sms, name.c_str());
   return buf;
 }
 
