@@ -210,7 +210,9 @@ typedef struct {
   int32_t spectral_tcgen05;/* 1: spectral step on tcgen05 (64-band plans, see
                               muffin_plan_set_spectral_kernel) */
   int32_t from_cache;      /* 1: taken from the in-process or file cache */
-  int32_t candidates;      /* configurations timed (0 when cached) */
+  int32_t candidates;      /* configurations considered (0 when cached); one
+                              that launches what the best so far launches is
+                              not timed */
   double ms_default;       /* one iteration of every chain group, default */
   double ms_best;          /* the same with the chosen variants */
   int32_t grad_chunk;      /* chosen gradient chunking (muffin_schedule) */

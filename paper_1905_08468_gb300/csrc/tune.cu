@@ -105,6 +105,28 @@ void apply(muffin_plan P, const Choice &c) {
   P->ana_pipe = c.ana_pipe;
 }
 
+// c without the choices that change no launch of this plan, so that candidates
+// with equal launches are not timed against one another
+Choice effective(muffin_plan P, Choice c) {
+  const bool wavelets = P->dict == 0;
+  c.dct_tc = P->L == 64 && P->p.precision == 0 ? c.dct_tc : 0;
+  if (P->spec_f32 || c.dct_tc) c.dct_ctas = 0;              // the dense kernel's grid
+  if (P->n == 32 || P->n == 64 || c.grad_chunk >= P->Cmax * P->Lt) c.grad_chunk = 0;   // one kernel
+  if (P->n < 128) c.fft_radix = 16;
+  if (!P->p.sure) c.group_order = 0;
+  if (!wavelets || P->J < 1) c.syn_packed = 0;
+  if (P->J < 2) c.syn_packed &= ~1;                         // bit 0: the coarse levels
+  c.ana_ring = 0;
+  if (!wavelets || P->J < 1 || P->n < 64) c.ana_pipe = 0;   // smaller levels: k_ana
+  return c;
+}
+
+bool same(const Choice &a, const Choice &b) {
+  return a.syn_packed == b.syn_packed && a.dct_ctas == b.dct_ctas && a.dct_tc == b.dct_tc &&
+         a.grad_chunk == b.grad_chunk && a.fft_radix == b.fft_radix &&
+         a.group_order == b.group_order && a.ana_ring == b.ana_ring && a.ana_pipe == b.ana_pipe;
+}
+
 // mean time of one iteration of every chain group with choice c
 muffin_status time_choice(muffin_plan P, const Choice &c, int reps, cudaEvent_t e0,
                           cudaEvent_t e1, double *ms) {
@@ -141,75 +163,62 @@ muffin_status tune(muffin_plan P, Choice *best, muffin_tune_info *info) {
   const double vox = (double)P->NL * P->Cmax * (P->p.sure ? 2 : 1);
   const int reps = vox >= 2e7 ? 3 : (vox >= 1e6 ? 5 : 10);
   Choice cur{};
-  const bool tf32 = P->p.precision == 0;   // a plan that asks for FP32 has no spectral choices
-  cur.dct_tc = P->L == 64 && tf32 ? 1 : 0; // the default kernel for 64 bands
+  cur.dct_tc = P->L == 64 && P->p.precision == 0 ? 1 : 0;   // the default kernel for 64 bands
   double t_def = 0.0, t_best = 0.0;
   int cand = 0;
   if (s == MUFFIN_OK) s = time_choice(P, cur, reps, e0, e1, &t_def);
   t_best = t_def;
   *best = cur;
   ++cand;
-  // coordinate search: synthesis variants, then the spectral grid
-  for (int v = 1; v <= 3 && s == MUFFIN_OK; ++v) {
+  // a candidate replaces the best where it is faster; one that launches what the
+  // best launches is counted, not timed (noise would choose between the two)
+  const auto consider = [&](const Choice &c) {
+    if (s != MUFFIN_OK) return;
+    ++cand;
+    if (same(effective(P, c), effective(P, *best))) return;
+    double t = 0.0;
+    s = time_choice(P, c, reps, e0, e1, &t);
+    if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
+  };
+  // coordinate search: synthesis variants, then the spectral kernel and its grid
+  for (int v = 1; v <= 3; ++v) {
     Choice c = *best;
     c.syn_packed = v;
-    double t = 0.0;
-    s = time_choice(P, c, reps, e0, e1, &t);
-    ++cand;
-    if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
+    consider(c);
   }
-  if (P->L == 64 && tf32 && s == MUFFIN_OK) {     // the other spectral kernel
+  if (cur.dct_tc) {                     // the other spectral kernel
     Choice c = *best;
     c.dct_tc = 0;
-    double t = 0.0;
-    s = time_choice(P, c, reps, e0, e1, &t);
-    ++cand;
-    if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
+    consider(c);
   }
-  for (int k = 1; k <= 2 && tf32 && s == MUFFIN_OK && !best->dct_tc; ++k) {
+  for (int k = 1; k <= 2 && P->p.precision == 0 && !best->dct_tc; ++k) {
     Choice c = *best;
     c.dct_ctas = k;
-    double t = 0.0;
-    s = time_choice(P, c, reps, e0, e1, &t);
-    ++cand;
-    if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
+    consider(c);
   }
   // the gradient's FFT passes over image chunks whose spectra fit in L2
   // (the images of one gradient call: C L of a chain group)
-  const int nimg = P->Cmax * P->Lt;
   for (int q : {48, 16}) {
-    if (q >= nimg || s != MUFFIN_OK) continue;
+    if (q >= P->Cmax * P->Lt) continue;
     Choice c = *best;
     c.grad_chunk = q;
-    double t = 0.0;
-    s = time_choice(P, c, reps, e0, e1, &t);
-    ++cand;
-    if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
+    consider(c);
   }
-  if (P->n >= 64 && s == MUFFIN_OK) {   // the radix-8 FFT plan
+  if (P->n >= 64) {                     // the radix-8 FFT plan
     Choice c = *best;
     c.fft_radix = 8;
-    double t = 0.0;
-    s = time_choice(P, c, reps, e0, e1, &t);
-    ++cand;
-    if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
+    consider(c);
   }
   // the other tile height of the analysis levels
-  if (P->J > 1 && P->dict == 0 && s == MUFFIN_OK) {
+  if (P->J > 0 && P->dict == 0) {
     Choice c = *best;
     c.ana_pipe = 1 - c.ana_pipe;
-    double t = 0.0;
-    s = time_choice(P, c, reps, e0, e1, &t);
-    ++cand;
-    if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
+    consider(c);
   }
-  for (int o = 1; o <= 2 && P->p.sure && s == MUFFIN_OK; ++o) {   // kernel order of the groups
+  for (int o = 1; o <= 2 && P->p.sure; ++o) {   // kernel order of the groups
     Choice c = *best;
     c.group_order = o;
-    double t = 0.0;
-    s = time_choice(P, c, reps, e0, e1, &t);
-    ++cand;
-    if (s == MUFFIN_OK && t < t_best) { t_best = t; *best = c; }
+    consider(c);
   }
   if (s == MUFFIN_OK) s = muffin::pi::leave(P, true);
   P->profiling = was_profiling;

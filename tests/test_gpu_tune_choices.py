@@ -16,6 +16,32 @@ def plan(pkg, n, L, **kw):
     return pkg.Plan(n, L, psf, **kw)
 
 
+@pytest.mark.parametrize("n,L,kw", [
+    (16, 2, {}), (16, 4, {}), (32, 16, {}), (32, 128, {}), (64, 32, {}), (64, 128, {}),
+    (32, 24, {}), (64, 8, {"precision": "fp32"}), (16, 16, {"dictionary": "iuwt"}),
+    (32, 4, {"levels": 1}), (16, 8, {"sure": True, "levels": 2})])
+def test_only_choices_with_an_effect_are_stored(tmp_path, n, L, kw):
+    cuda()
+    import paper_1905_08468_gb300 as pkg
+    cache = tmp_path / "tune.txt"
+    with plan(pkg, n, L, **kw) as p:
+        assert p.autotune(str(cache)).from_cache == 0
+    syn, ctas, tc, chunk, radix, order, ring, pipe = map(int, cache.read_text().split()[2:])
+    if L & (L - 1) == 0:
+        assert ctas == 0 and tc == 0                 # the fast DCT has no variants
+    assert radix == 16 and ring == 0                 # one plan below 128 pixels a side
+    if n in (32, 64):
+        assert chunk == 0                            # the gradient is one kernel
+    if kw.get("dictionary") == "iuwt":
+        assert syn == 0 and pipe == 0
+    if kw.get("levels") == 1:
+        assert syn & 1 == 0                          # no coarse level
+    if n < 64:
+        assert pipe == 0                             # no level of the columns kernel
+    if not kw.get("sure"):
+        assert order == 0
+
+
 def test_lines_of_earlier_kernels_are_not_used(tmp_path):
     cuda()
     import paper_1905_08468_gb300 as pkg
