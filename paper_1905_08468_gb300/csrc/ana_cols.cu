@@ -60,6 +60,7 @@ struct Tile {
   static constexpr int GRP = 40 / NG;         // chunks of a group
   static constexpr int VB = 2 * CY * VP;      // floats of a buffer: low rows, high rows
   static_assert(ITEMS <= NT && 4 * GRP * NG == VP, "an item a thread, whole rows");
+  static_assert(CX == 64 && CY >= 8 && ITEMS == 128, "ana_mask_words");
 };
 
 enum Source { SRC_ITERATE, SRC_OPERATOR, SRC_LL };

@@ -44,6 +44,7 @@ constexpr int IY = 32, IX = 128, INT = 160;   // output tile, threads (a column 
 constexpr int VP = INT;                       // floats of a smoothed row
 constexpr int RB = 8;                         // rows whose U is in flight
 static_assert(IX + 4 * 8 <= INT, "a column of the tile and its widest halo a thread");
+static_assert(IX == 128 && IY == 32, "iuwt_mask_words");
 
 // B3 spline tap m of [1 4 6 4 1] / 16
 __device__ __forceinline__ constexpr float b3(int m) {

@@ -92,8 +92,8 @@ int set_last_error_code(int s, const char *msg);
 // FP32 gradient pipeline: g[c][l] = H_l^T H_l x[c][l] - (c == 0 && b ? b[l] : 0)
 // for nimg = C*L images.  S: spectrum scratch [nimg][n/2+1][n] float2.
 // kspec: [L][n/2+1][n] = |h_hat_l(ky, kx)|^2 / n^2 (kx-major).
-// chunk > 0: the three passes run over `chunk` images at a time (S then
-// needs room for chunk images only and stays in L2 between the passes);
+// chunk > 0: the three passes run over `chunk` images at a time (the
+// part of S that is used stays in L2 between the passes);
 // chunk <= 0: each pass over all images at once.
 // radix 16 (default) or 8 (n >= 128): the largest radix of the row passes; tw
 // must hold that plan's twiddle tables (fft32_tables with the same radix).
@@ -228,6 +228,28 @@ cudaError_t upload_filters(const double h[8][16]);
 
 enum WaveMode { WAVE_TRANSFORM = 0, WAVE_ITERATE = 1 };
 
+// Words (32 bits) a band that the primal's launch of a level writes for the
+// derivatives' (the largest of the levels, level 1, and of both tile heights):
+// ana_cols.cu stores 128 a tile of 64 x 8 coefficients and basis, iuwt.cu two a
+// column of a tile of 32 x 128 pixels, whole tiles where the image ends inside one.
+constexpr size_t ana_mask_words(int n, int K) {
+  return n < 64 ? 0 : (size_t)((n / 2 + 63) / 64) * ((n / 2 + 7) / 8) * 128 * K;
+}
+constexpr size_t iuwt_mask_words(int n) {
+  return (size_t)((n + 127) / 128) * ((n + 31) / 32) * (n < 128 ? n : 128) * 2;
+}
+constexpr size_t mask_words(int n, int K) {
+  return ana_mask_words(n, K) > iuwt_mask_words(n) ? ana_mask_words(n, K) : iuwt_mask_words(n);
+}
+// they borrow the spectra of a band's three chains
+constexpr bool masks_fit() {
+  for (int n = 2; n <= 2048; n *= 2)
+    if (mask_words(n, 8) * sizeof(uint32_t) > (size_t)3 * (n / 2 + 1) * n * sizeof(float2))
+      return false;
+  return true;
+}
+static_assert(masks_fit(), "the masks fit in the gradient's spectra at every size");
+
 struct WaveArgs {
   int n, L, K, J, C;       // L = all bands of all cubes of the batch
   int Lc;                  // bands per cube (0: one cube of L bands)
@@ -236,8 +258,8 @@ struct WaveArgs {
   float *scratch;          // LL scratch: level j (1 <= j < J) holds
                            // [C][L][K][n>>j][n>>j] at scratch + lvl_off[j]
   size_t lvl_off[16];
-  uint32_t *masks;         // three chains: masks of the level-1 duals, n^2 K / 8 bytes a
-                           // band (the gradient's spectrum scratch, free by then)
+  uint32_t *masks;         // three chains: the primal's masks, mask_words(n, K) a band
+                           // (the gradient's spectrum scratch, free by then)
   int dict;                // 0: union of K Daubechies bases, 1: IUWT (K = J + 1 planes)
   int ana_pipe;            // analysis: 1 takes the other tile height than the rule's
   int syn_packed;          // synthesis variant: bit 0 coarse levels, bit 1
