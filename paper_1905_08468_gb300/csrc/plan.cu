@@ -145,6 +145,13 @@ bool spectral_f32(const muffin_params *p) {
   const int L = p->nbands;
   return p->precision == 1 || (L >= 2 && L <= 1024 && L != 64 && (L & (L - 1)) == 0);
 }
+// Which tables a plan keeps beside those of the fast DCT: with 64 bands (all of
+// them, 80 KB) the TF32 halves of C and C^T for tcgen05 and the folded ones for the DCT
+// operator and the other spectral kernel; else the folded ones where the dense kernel
+// runs.  L x L tables that nothing reads cost 20 MB and 1.5 ms of a plan's creation
+// at 1024 bands.
+bool tf32_tables(const muffin_params *p) { return p->nbands == 64; }
+bool fold_tables(const muffin_params *p) { return p->nbands == 64 || !spectral_f32(p); }
 
 // copy a caller array (host or device) into dst (device), count floats
 muffin_status fetch(muffin_plan P, const float *src, float *dst, size_t count) {
@@ -387,11 +394,13 @@ muffin_status plan_alloc_init(muffin_plan P, const float *alpha, const float *be
   CK(P->alloc(&P->tw32, tw_len + fft32_cols_table_len(n)));
   CK(P->alloc(&P->tw64, (size_t)n));
   const size_t LL2 = (size_t)P->Lp * P->Lp;
-  CK(P->alloc(&P->chi, LL2));
-  CK(P->alloc(&P->clo, LL2));
-  CK(P->alloc(&P->cthi, LL2));
-  CK(P->alloc(&P->ctlo, LL2));
-  CK(P->alloc(&P->fold, (size_t)dct_fold_table_len(L)));
+  if (tf32_tables(&P->p)) {
+    CK(P->alloc(&P->chi, LL2));
+    CK(P->alloc(&P->clo, LL2));
+    CK(P->alloc(&P->cthi, LL2));
+    CK(P->alloc(&P->ctlo, LL2));
+  }
+  if (fold_tables(&P->p)) CK(P->alloc(&P->fold, (size_t)dct_fold_table_len(L)));
   if (P->spec_f32) {
     P->ftw_len = dct_f32_table_len(L) - L;
     CK(P->alloc(&P->ftab, (size_t)dct_f32_table_len(L)));
@@ -469,25 +478,31 @@ muffin_status plan_alloc_init(muffin_plan P, const float *alpha, const float *be
   for (int p = 1; p <= 8; ++p) daubechies_lowpass(p, taps[p - 1]);
   CK(upload_filters(taps));
 
-  // ---- DCT tables, TF32 hi/lo split, zero padded to Lp
-  std::vector<double> C((size_t)L * L);
-  dct2_matrix(L, C.data());
-  const int Lp = P->Lp;
-  std::vector<float> hi(LL2, 0.f), lo(LL2, 0.f), thi(LL2, 0.f), tlo(LL2, 0.f);
-  for (int k = 0; k < L; ++k)
-    for (int l = 0; l < L; ++l) {
-      const float c = (float)C[(size_t)k * L + l];
-      const float h = tf32_round(c), r = tf32_round(c - h);
-      hi[(size_t)k * Lp + l] = h; lo[(size_t)k * Lp + l] = r;
-      thi[(size_t)l * Lp + k] = h; tlo[(size_t)l * Lp + k] = r;
-    }
-  CK(cudaMemcpyAsync(P->chi, hi.data(), LL2 * 4, cudaMemcpyHostToDevice, P->ws));
-  CK(cudaMemcpyAsync(P->clo, lo.data(), LL2 * 4, cudaMemcpyHostToDevice, P->ws));
-  CK(cudaMemcpyAsync(P->cthi, thi.data(), LL2 * 4, cudaMemcpyHostToDevice, P->ws));
-  CK(cudaMemcpyAsync(P->ctlo, tlo.data(), LL2 * 4, cudaMemcpyHostToDevice, P->ws));
-  std::vector<float> fold((size_t)dct_fold_table_len(L));
-  dct_fold_tables(L, C.data(), fold.data());
-  CK(cudaMemcpyAsync(P->fold, fold.data(), fold.size() * 4, cudaMemcpyHostToDevice, P->ws));
+  // ---- DCT tables (the host arrays outlive the copies: synchronised below)
+  std::vector<double> C;
+  if (fold_tables(&P->p)) {
+    C.resize((size_t)L * L);
+    dct2_matrix(L, C.data());
+  }
+  std::vector<float> fold(C.empty() ? 0 : (size_t)dct_fold_table_len(L)), tf[4];
+  if (!fold.empty()) {
+    dct_fold_tables(L, C.data(), fold.data());
+    CK(cudaMemcpyAsync(P->fold, fold.data(), fold.size() * 4, cudaMemcpyHostToDevice, P->ws));
+  }
+  if (tf32_tables(&P->p)) {            // C and C^T split in TF32 hi + lo
+    const int Lp = P->Lp;
+    for (std::vector<float> &t : tf) t.assign(LL2, 0.f);
+    for (int k = 0; k < L; ++k)
+      for (int l = 0; l < L; ++l) {
+        const float c = (float)C[(size_t)k * L + l];
+        const float h = tf32_round(c), r = tf32_round(c - h);
+        tf[0][(size_t)k * Lp + l] = h; tf[1][(size_t)k * Lp + l] = r;
+        tf[2][(size_t)l * Lp + k] = h; tf[3][(size_t)l * Lp + k] = r;
+      }
+    float *const to[4] = {P->chi, P->clo, P->cthi, P->ctlo};
+    for (int m = 0; m < 4; ++m)
+      CK(cudaMemcpyAsync(to[m], tf[m].data(), LL2 * 4, cudaMemcpyHostToDevice, P->ws));
+  }
   std::vector<float2> ft(P->spec_f32 ? (size_t)dct_f32_table_len(L) : 0);
   if (P->spec_f32) {
     dct_f32_tables(L, ft.data());
@@ -837,14 +852,17 @@ size_t estimate_bytes(const muffin_params *p) {
   else
     for (int j = 1; j < p->levels; ++j) ll += C * Lt * K * (n >> j) * (n >> j);
   size_t b = 3 * NL * 16 + Lt * nh * n * 4 + (size_t)(fft32_table_len((int)n, 16) + fft32_table_len((int)n, 8) + fft32_cols_table_len((int)n)) * 8 + n * 16 +
-             4 * Lp * Lp * 4 + (size_t)dct_fold_table_len((int)L) * 4 + B * N * 4 + Lt * 4 + B * sizeof(DevScalars) + B * 32 + 4 + 4 +
+             B * N * 4 + Lt * 4 + B * sizeof(DevScalars) + B * 32 + 4 + 4 +
              (kRedSure + 65 * Lt + 6 * (Lt > 4096 ? Lt : 4096)) * 8 + Lt * 8 + Lt * sizeof(ImageStat) + Lt * 8 + n * 16 +
              C * Lt * nh * n * 8 + (ll ? ll : 1) * 4 + 3 * NL * 4 +
              C * NL * (5 + K) * 4;
   if (p->sure) b += 3 * NL * (5 + K) * 4 + 2 * NL * 4 + C * Lt * nh * n * 8 + (ll ? ll : 1) * 4;
   b += monitor_scratch_doubles((int)Lt) * 8;
+  // 16 bytes of slack per allocation
   if (spectral_f32(p)) b += (size_t)dct_f32_table_len((int)L) * 8 + 16;
-  return b + (p->sure ? 44 : 34) * 16;   // 16 bytes of slack per allocation
+  if (fold_tables(p)) b += (size_t)dct_fold_table_len((int)L) * 4 + 16;
+  if (tf32_tables(p)) b += 4 * (Lp * Lp * 4 + 16);
+  return b + (p->sure ? 39 : 29) * 16;
 }
 
 muffin_status create(const muffin_params *p, const float *psf, const float *alpha,
