@@ -12,9 +12,9 @@
 //
 // S_j is the separable B3 spline [1 4 6 4 1]/16 dilated by D = 2^j with periodic
 // boundaries.  One launch per scale and set of chains, specialised on D: a lane
-// owns one column of a 32 x 128 tile and its 2 D halo rows in registers (loaded
-// coalesced along the rows), smooths it along y there and puts the smoothed rows
-// into shared memory; after one barrier it smooths along x (five conflict-free
+// owns one column of a 32 x 128 tile (8 x 128 where there are few) and its 2 D halo
+// rows in registers (loaded coalesced along the rows), smooths it along y there and
+// puts the smoothed rows into shared memory; after one barrier it smooths along x (five conflict-free
 // reads a pixel) and does the scale's dual update (analysis) or Horner step
 // (synthesis) on its own column, whose unsmoothed values it still holds.  U is
 // requested eight rows ahead.  The running image of the next scale goes to a
@@ -28,7 +28,7 @@
 // rows ahead, and into L2 by the whole CTA first: 295 without).
 //
 // One chain a CTA: the primal's launch leaves its masks (Pi(p) per coefficient,
-// U(m) per pixel: a word of 32 rows a lane and plane) for the derivatives'.
+// U(m) per pixel: a word a lane, tile and plane) for the derivatives'.
 #include <cuda_runtime.h>
 
 #include <stdint.h>
@@ -40,11 +40,11 @@ namespace muffin {
 
 namespace {
 
-constexpr int IY = 32, IX = 128, INT = 160;   // output tile, threads (a column each)
+constexpr int IX = 128, INT = 160;            // output tile's columns, threads (a column each)
 constexpr int VP = INT;                       // floats of a smoothed row
 constexpr int RB = 8;                         // rows whose U is in flight
 static_assert(IX + 4 * 8 <= INT, "a column of the tile and its widest halo a thread");
-static_assert(IX == 128 && IY == 32, "iuwt_mask_words");
+static_assert(IX == 128, "iuwt_mask_words");
 
 // B3 spline tap m of [1 4 6 4 1] / 16
 __device__ __forceinline__ constexpr float b3(int m) {
@@ -68,7 +68,7 @@ struct IuwtArgs {
 
 // y smoothing of the lane's column into shared memory, then (after the barrier)
 // x smoothing of row r at the lane's own pixel
-template <int D>
+template <int D, int IY>
 __device__ __forceinline__ void smooth_y(const float (&c)[IY + 4 * D], float *v) {
 #pragma unroll
   for (int r = 0; r < IY; ++r) {
@@ -91,7 +91,7 @@ struct Place {
   int lane;                      // column of the tile (halo: < 0 or >= IX)
   bool own;                      // a pixel column of the image
 };
-template <int D>
+template <int D, int IY>
 __device__ __forceinline__ Place place(int n) {
   Place q;
   const int ntx = (n + IX - 1) / IX;
@@ -104,6 +104,7 @@ __device__ __forceinline__ Place place(int n) {
 }
 
 // the tile's rows of an image into L2: a 128-byte line a thread and round
+template <int IY>
 __device__ __forceinline__ void prefetch_tile(const float *img, unsigned n, unsigned y0) {
   const int ntx = (n + IX - 1) / IX;
   const unsigned x0 = (blockIdx.x % ntx) * IX;
@@ -115,13 +116,13 @@ __device__ __forceinline__ void prefetch_tile(const float *img, unsigned n, unsi
 
 // chain c = 0 (DERIV = false; masks recorded where a.masks is set), or
 // 1 + blockIdx.z
-template <int MODE, int D, bool LAST, bool DERIV>
+template <int MODE, int D, bool LAST, bool DERIV, int IY>
 __global__ void __launch_bounds__(INT, 3) k_iuwt_ana(IuwtArgs a) {
   chain_enter();
   __shared__ float vs[IY * VP];
   const unsigned n = a.n, nm = n - 1;
   const int l = blockIdx.y, c = DERIV ? 1 + blockIdx.z : 0, tid = threadIdx.x;
-  const Place w = place<D>(n);
+  const Place w = place<D, IY>(n);
   const size_t NN = (size_t)n * n, CS = (size_t)a.L * NN;
   float mu = 0.f, q = 1.f;
   if (MODE == WAVE_ITERATE) {
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(INT, 3) k_iuwt_ana(IuwtArgs a) {
         col[i] = fmaf(mu, col[i], 2.f * xt[o] - x[o]);
       }
     }
-    smooth_y<D>(col, vs + tid);
+    smooth_y<D, IY>(col, vs + tid);
   }
   constexpr int NP = LAST ? 2 : 1;
   float *uj = a.u + ((size_t)(c * a.L + l) * a.P + a.j) * NN + (size_t)w.y0 * n + w.xx;
@@ -210,13 +211,13 @@ __global__ void __launch_bounds__(INT, 3) k_iuwt_ana(IuwtArgs a) {
 // TOP: the coarsest step (source P_J - P_{J-1}); otherwise the running image of
 // scale j + 1.  Scales j > 0 take chains blockIdx.z; j = 0 (D = 1) ends in the
 // prox, chain 0 or chains 1 + blockIdx.z.
-template <int MODE, int D, bool TOP, bool DERIV>
+template <int MODE, int D, bool TOP, bool DERIV, int IY>
 __global__ void __launch_bounds__(INT, 3) k_iuwt_syn(IuwtArgs a) {
   chain_enter();
   __shared__ float vs[IY * VP];
   const unsigned n = a.n, nm = n - 1;
   const int l = blockIdx.y, c = (DERIV ? 1 : 0) + blockIdx.z, tid = threadIdx.x;
-  const Place w = place<D>(n);
+  const Place w = place<D, IY>(n);
   const size_t NN = (size_t)n * n, CS = (size_t)a.L * NN, US = CS * a.P;
   // chain 1's W^T u + mu W^T u'_mu (Algorithm 3) by linearity, from mixed inputs
   const bool mix = D == 1 && DERIV && c == 1;
@@ -224,10 +225,10 @@ __global__ void __launch_bounds__(INT, 3) k_iuwt_syn(IuwtArgs a) {
   const float *ub = (MODE == WAVE_TRANSFORM ? a.in : a.ur) + c * US + (size_t)l * a.P * NN;
   if (D == 1 && MODE == WAVE_ITERATE) {
     const size_t o = c * CS + l * NN;
-    prefetch_tile(ub, n, w.y0);
-    prefetch_tile(a.x + o, n, w.y0);
-    prefetch_tile(a.g + o, n, w.y0);
-    prefetch_tile(a.t + o, n, w.y0);
+    prefetch_tile<IY>(ub, n, w.y0);
+    prefetch_tile<IY>(a.x + o, n, w.y0);
+    prefetch_tile<IY>(a.g + o, n, w.y0);
+    prefetch_tile<IY>(a.t + o, n, w.y0);
   }
   float col[IY + 4 * D];
   if (tid < IX + 4 * D) {
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(INT, 3) k_iuwt_syn(IuwtArgs a) {
         col[i] = fmaf(mu, col[i], TOP ? s1[o] - s2[o] : s1[o]);
       }
     }
-    smooth_y<D>(col, vs + tid);
+    smooth_y<D, IY>(col, vs + tid);
   }
   __syncthreads();
   if (!w.own) return;
@@ -284,7 +285,8 @@ __global__ void __launch_bounds__(INT, 3) k_iuwt_syn(IuwtArgs a) {
     const float bl = MODE == WAVE_ITERATE ? a.beta[l] : 0.f;
     const float sc = c == 1 ? bl : bl * mu;          // mu_l, beta_l, mu_l
     const size_t i1 = c * CS + l * NN + i0;
-    constexpr int RQ = 2;                            // four arrays a row: 2 x 2 rows in flight
+    // four arrays a row: 2 x 2 rows in flight, or all of a low tile's
+    constexpr int RQ = IY == 8 ? 8 : 2;
     float in[2][4][RQ];
     auto request = [&](int r0, float (&v)[4][RQ]) {
 #pragma unroll
@@ -331,30 +333,54 @@ __global__ void __launch_bounds__(INT, 3) k_iuwt_syn(IuwtArgs a) {
   }
 }
 
-inline int itiles(int n) { return ((n + IX - 1) / IX) * ((n + IY - 1) / IY); }
+inline int itiles(int n, int rows) { return ((n + IX - 1) / IX) * ((n + rows - 1) / rows); }
 
-template <int CH, int MODE, int D>
-void launch_ana_d(const IuwtArgs &a, cudaStream_t st) {
-  const dim3 g(itiles(a.n), a.L), g2(itiles(a.n), a.L, 2);
+// Tiles of 8 rows while those of 32 fill less than a wave (3 CTAs on 152 SMs, one
+// chain).  A lane walks its rows one after the other, two at a time in the prox, and
+// with few CTAs nothing covers that walk: below a wave four times the CTAs with a
+// quarter of it, all rows in flight at once, are faster at every size, number of
+// scales and number of chains (an iteration of a plain solve, one scale: 32 x 32 x 8 30.9
+// -> 18.5 us, 64 x 64 x 32 34.5 -> 21.8, 256 x 256 x 24 51 -> 46; four scales, 128 x 128 x
+// 100, 400 tiles: 137 -> 133; three chains 256 x 256 x 16, 489 -> 430).  The lead shrinks
+// towards a wave, where the CTAs cover each other and the halo of a low tile (32 rows
+// at the widest beside its 8) is what is left of the difference.
+inline bool low_tiles(const IuwtArgs &a) { return (long long)itiles(a.n, 32) * a.L < 3 * 152; }
+
+template <int CH, int MODE, int D, int IY>
+void launch_ana_y(const IuwtArgs &a, cudaStream_t st) {
+  const dim3 g(itiles(a.n, IY), a.L), g2(itiles(a.n, IY), a.L, 2);
   if (a.j == a.J - 1) {
-    launch_chain(k_iuwt_ana<MODE, D, true, false>, g, INT, 0, st, a);
-    if constexpr (CH == 3) launch_chain(k_iuwt_ana<MODE, D, true, true>, g2, INT, 0, st, a);
+    launch_chain(k_iuwt_ana<MODE, D, true, false, IY>, g, INT, 0, st, a);
+    if constexpr (CH == 3) launch_chain(k_iuwt_ana<MODE, D, true, true, IY>, g2, INT, 0, st, a);
   } else {
-    launch_chain(k_iuwt_ana<MODE, D, false, false>, g, INT, 0, st, a);
-    if constexpr (CH == 3) launch_chain(k_iuwt_ana<MODE, D, false, true>, g2, INT, 0, st, a);
+    launch_chain(k_iuwt_ana<MODE, D, false, false, IY>, g, INT, 0, st, a);
+    if constexpr (CH == 3) launch_chain(k_iuwt_ana<MODE, D, false, true, IY>, g2, INT, 0, st, a);
+  }
+}
+
+template <int CH, int MODE, int D, int IY>
+void launch_syn_y(const IuwtArgs &a, cudaStream_t st) {
+  const bool top = a.j == a.J - 1;
+  const int nt = itiles(a.n, IY);
+  const dim3 g(nt, a.L, D > 1 ? CH : 1), g2(nt, a.L, 2);
+  if (top) launch_chain(k_iuwt_syn<MODE, D, true, false, IY>, g, INT, 0, st, a);
+  else launch_chain(k_iuwt_syn<MODE, D, false, false, IY>, g, INT, 0, st, a);
+  if constexpr (CH == 3 && D == 1) {
+    if (top) launch_chain(k_iuwt_syn<MODE, D, true, true, IY>, g2, INT, 0, st, a);
+    else launch_chain(k_iuwt_syn<MODE, D, false, true, IY>, g2, INT, 0, st, a);
   }
 }
 
 template <int CH, int MODE, int D>
+void launch_ana_d(const IuwtArgs &a, cudaStream_t st) {
+  if (low_tiles(a)) launch_ana_y<CH, MODE, D, 8>(a, st);
+  else launch_ana_y<CH, MODE, D, 32>(a, st);
+}
+
+template <int CH, int MODE, int D>
 void launch_syn_d(const IuwtArgs &a, cudaStream_t st) {
-  const bool top = a.j == a.J - 1;
-  const dim3 g(itiles(a.n), a.L, D > 1 ? CH : 1), g2(itiles(a.n), a.L, 2);
-  if (top) launch_chain(k_iuwt_syn<MODE, D, true, false>, g, INT, 0, st, a);
-  else launch_chain(k_iuwt_syn<MODE, D, false, false>, g, INT, 0, st, a);
-  if constexpr (CH == 3 && D == 1) {
-    if (top) launch_chain(k_iuwt_syn<MODE, D, true, true>, g2, INT, 0, st, a);
-    else launch_chain(k_iuwt_syn<MODE, D, false, true>, g2, INT, 0, st, a);
-  }
+  if (low_tiles(a)) launch_syn_y<CH, MODE, D, 8>(a, st);
+  else launch_syn_y<CH, MODE, D, 32>(a, st);
 }
 
 template <int CH, int MODE>

@@ -231,12 +231,12 @@ enum WaveMode { WAVE_TRANSFORM = 0, WAVE_ITERATE = 1 };
 // Words (32 bits) a band that the primal's launch of a level writes for the
 // derivatives' (the largest of the levels, level 1, and of both tile heights):
 // ana_cols.cu stores 128 a tile of 64 x 8 coefficients and basis, iuwt.cu two a
-// column of a tile of 32 x 128 pixels, whole tiles where the image ends inside one.
+// column of a tile of 8 x 128 pixels, whole tiles where the image ends inside one.
 constexpr size_t ana_mask_words(int n, int K) {
   return n < 64 ? 0 : (size_t)((n / 2 + 63) / 64) * ((n / 2 + 7) / 8) * 128 * K;
 }
 constexpr size_t iuwt_mask_words(int n) {
-  return (size_t)((n + 127) / 128) * ((n + 31) / 32) * (n < 128 ? n : 128) * 2;
+  return (size_t)((n + 127) / 128) * ((n + 7) / 8) * (n < 128 ? n : 128) * 2;
 }
 constexpr size_t mask_words(int n, int K) {
   return ana_mask_words(n, K) > iuwt_mask_words(n) ? ana_mask_words(n, K) : iuwt_mask_words(n);
