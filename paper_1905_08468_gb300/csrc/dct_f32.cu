@@ -18,8 +18,8 @@
 // shared-memory Stockham transforms of the gradient passes.  The work is
 // O(L log L) per pixel, so the step is bound by its HBM traffic at every L
 // (512 x 512 x 256, one chain: 0.28 ms, 4.8 TB/s; the dense 3xTF32 product on
-// mma.sync took 1.74 ms).  Images with few tiles run 64-thread CTAs with a
-// quarter of the pixels (64 x 64 x 32, three chains: 24.8 -> 17.6 us).  The old
+// mma.sync took 1.74 ms).  Where tiles are few, 64-thread CTAs take a quarter of the
+// pixels (64 x 64 x 32, three chains: 24.8 -> 17.6 us).  The old
 // duals of a chain are requested before the chain's forward DFT (512 x 512 x
 // 32, three chains: 165 -> 134 us), and chain 2's gamma v'_gamma + v is formed
 // after the inverse DFTs, which are linear, so no dual stays in a register.
@@ -299,10 +299,16 @@ cudaError_t launch_f32_t(const F32Args &a, cudaStream_t st, Prof *prof) {
 template <int L, int CH, int MODE>
 cudaError_t launch_f32(const F32Args &a, cudaStream_t st, Prof *prof) {
   const size_t tiles = (a.npix + FShape<L, 256>::PT - 1) / FShape<L, 256>::PT * a.B;
-  // below a 256-thread CTA an SM the quarter-size tiles fill the chip better
-  // (64 x 64 x 32, three chains: 24.8 -> 18 us); from there on the wide tiles' longer
-  // rows win (256 x 256 x 32, three chains, 256 tiles: 43.7 against 35.1 us)
-  return tiles < 150 ? launch_f32_t<L, CH, MODE, 64>(a, st, prof)
+  // 64-thread CTAs (quarter-size tiles) where the 256-thread ones are too few.  Up to
+  // 128 bands below one an SM they fill the chip better (64 x 64 x 32, three chains:
+  // 24.8 -> 18 us; from there on the wide tiles' longer rows win, 256 x 256 x 32: 43.7
+  // against 35.1).  Short spectra have too little work a thread for it (8 bands, one
+  // chain: 8.2 against 7.0 us; 64 x 64 x 16, three: 15.4 against 12.6), and long ones
+  // tables that every CTA loads (32 x 32 x 1024, 128 wide tiles: 34.7 against 14.2
+  // us; 64 x 64 x 256: 12.8 against 11.4), so the line lies lower there.
+  constexpr size_t few = CH == 3 ? (L <= 16 ? 0 : L <= 128 ? 150 : 76)
+                                 : (L < 16 || L == 1024 ? 0 : L <= 128 ? 150 : L == 256 ? 76 : 38);
+  return tiles < few ? launch_f32_t<L, CH, MODE, 64>(a, st, prof)
                      : launch_f32_t<L, CH, MODE, 256>(a, st, prof);
 }
 
