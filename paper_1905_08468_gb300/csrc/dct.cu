@@ -62,11 +62,12 @@ __device__ __forceinline__ void st4(float *p, float4 v) {
   *reinterpret_cast<float4 *>(p) = v;
 }
 
-// acc[r] (4 pixels) += sum_j A[j * Mp + r] * B[j * PT], j < len, r < R
-template <int PT, int R>
+// acc[r] (4 pixels) += sum_j A[j * Mp + r] * B[j * PT], j < len, r < R; U steps' loads
+// in flight
+template <int PT, int R, int U>
 __device__ __forceinline__ void half_product(const float *__restrict__ A, int Mp, const float *B,
                                              int len, float2 (&acc)[R][2]) {
-#pragma unroll 4
+#pragma unroll U
   for (int j = 0; j < len; ++j) {
     float cr[R];
     if constexpr (R == 4) {
@@ -87,8 +88,8 @@ __device__ __forceinline__ void half_product(const float *__restrict__ A, int Mp
   }
 }
 
-// RB: rows of a task of C^T v
-template <int CH, int MODE, int PT, int RB>
+// RB: rows of a task of C^T v; U: depth of the products' loads
+template <int CH, int MODE, int PT, int RB, int U>
 __global__ void __launch_bounds__(DT, 3) k_dct_fold(FoldArgs a) {
   chain_enter();
   constexpr int PG = PT / 4;                      // pixel groups
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(DT, 3) k_dct_fold(FoldArgs a) {
           float2 acc[RK][2];
 #pragma unroll
           for (int r = 0; r < RK; ++r) acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
-          half_product<PT, RK>(a.fwd + (size_t)par * Mp * Mp + r0, Mp,
+          half_product<PT, RK, U>(a.fwd + (size_t)par * Mp * Mp + r0, Mp,
                            zs + (2 * c + par) * half + 4 * pg, len, acc);
           const float sg = c == 2 ? sigma : sigma * gamma;
 #pragma unroll
@@ -224,8 +225,8 @@ __global__ void __launch_bounds__(DT, 3) k_dct_fold(FoldArgs a) {
       float2 ev[RB][2], od[RB][2];
 #pragma unroll
       for (int r = 0; r < RB; ++r) ev[r][0] = ev[r][1] = od[r][0] = od[r][1] = make_float2(0.f, 0.f);
-      half_product<PT, RB>(a.bwd + r0, Mp, vc, M, ev);
-      half_product<PT, RB>(a.bwd + (size_t)Mp * Mp + r0, Mp, vc + half, Mo, od);
+      half_product<PT, RB, U>(a.bwd + r0, Mp, vc, M, ev);
+      half_product<PT, RB, U>(a.bwd + (size_t)Mp * Mp + r0, Mp, vc + half, Mo, od);
       if (!ok) continue;
       const float g = c == 2 ? 1.f : gamma;
       float s2[4];
@@ -248,19 +249,23 @@ __global__ void __launch_bounds__(DT, 3) k_dct_fold(FoldArgs a) {
   }
 }
 
-template <int CH, int MODE, int PT, int RB>
+template <int CH, int MODE, int PT, int RB, int U = 4>
 cudaError_t launch_fold_r(FoldArgs &a, int ctas_per_sm, size_t sm, cudaStream_t st, Prof *prof) {
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_dct_fold<CH, MODE, PT, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_dct_fold<CH, MODE, PT, RB, U>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          208 * 1024);
     attr = true;
   }
   a.tiles_per_cube = (int)((a.npix + PT - 1) / PT);
   a.ntiles = a.tiles_per_cube * a.B;
   // threads: whole row groups of C z in as few rounds as 256 threads allow,
-  // all of them busy in every round (37 bands: 160 threads, one round)
-  const int groups = 2 * (a.Mp / RK), rounds = (groups * (PT / 4) + DT - 1) / DT;
+  // all of them busy in every round (37 bands: 160 threads, one round); narrow tiles,
+  // which are few, take as many as load the tile in a round and as C^T v of all
+  // chains has (64 x 64 x 20, three chains: 17.1 -> 12.7 us)
+  int groups = 2 * (a.Mp / RK);
+  if (PT == 16) groups = std::max(groups, std::max(std::min(a.M, 32), RB == 2 ? CH * (a.Mp / RB) : 0));
+  const int rounds = (groups * (PT / 4) + DT - 1) / DT;
   const int threads = ((groups + rounds - 1) / rounds * (PT / 4) + 31) / 32 * 32;
   int grid = a.ntiles;
   if (ctas_per_sm > 0) {
@@ -273,7 +278,7 @@ cudaError_t launch_fold_r(FoldArgs &a, int ctas_per_sm, size_t sm, cudaStream_t 
   ProfScope ps(prof, MODE == WAVE_ITERATE ? "spectral_dual" : "spectral_op",
                MODE == WAVE_ITERATE ? CH * vox * 20.0 : vox * 8.0,
                (MODE == WAVE_ITERATE ? 2.0 : 1.0) * CH * a.L * vox, st);
-  launch_chain(k_dct_fold<CH, MODE, PT, RB>, grid, threads, sm, st, a);
+  launch_chain(k_dct_fold<CH, MODE, PT, RB, U>, grid, threads, sm, st, a);
   return cudaGetLastError();
 }
 
@@ -286,20 +291,43 @@ cudaError_t launch_fold(FoldArgs &a, int ctas_per_sm, size_t sm, cudaStream_t st
                   : launch_fold_r<CH, MODE, PT, 4>(a, ctas_per_sm, sm, st, prof);
 }
 
+// Tiles of 16 pixels.  Few of them are bound by the latency of a thread's tasks, so an
+// iteration's step takes the short ones (two rows) up to 200 bands (64 x 64 x 56, one
+// chain 13.8 -> 12.4 us), with three chains up to 64 (64 x 64 x 48: 24.8 -> 16.3).  From
+// 200 bands on the tables (4 Mp^2 floats, 160 KB) stay in no L1, and the loads of eight
+// steps in flight cover L2's latency (128 x 128 x 250 with the line below: 160 -> 120
+// us; from 300 on with four rows a task, 64 x 64 x 1000: 1000 -> 919).
+template <int CH, int MODE>
+cudaError_t launch_narrow(FoldArgs &a, int ctas_per_sm, size_t sm, cudaStream_t st, Prof *prof) {
+  if constexpr (MODE == WAVE_ITERATE) {
+    if (a.L < (CH == 1 ? 200 : 64)) return launch_fold_r<CH, MODE, 16, 2>(a, ctas_per_sm, sm, st, prof);
+    if constexpr (CH == 1) {
+      if (a.L < 260) return launch_fold_r<CH, MODE, 16, 2, 8>(a, ctas_per_sm, sm, st, prof);
+      if (a.L >= 300) return launch_fold_r<CH, MODE, 16, 4, 8>(a, ctas_per_sm, sm, st, prof);
+    }
+  }
+  return launch_fold<CH, MODE, 16>(a, ctas_per_sm, sm, st, prof);
+}
+
 template <int CH, int MODE>
 cudaError_t dispatch_fold(FoldArgs &a, int ctas_per_sm, cudaStream_t st, Prof *prof) {
   // The widest pixel tile with room for three CTAs an SM (wider rows for the
   // loads and more products per coefficient read), narrower while the image
-  // has too few tiles for two CTAs an SM.
+  // has too few tiles for two CTAs an SM.  One chain of 200 bands and more, whose
+  // tables leave no L1 beside wide tiles, goes on with narrow ones until the wide
+  // ones' second wave is a third full (608 of them: 128 x 128 x 250, 512 tiles of 32
+  // pixels, 160 -> 120 us; 256 x 256 x 200, 2048: wide 256, narrow 275).
   const auto sm = [&](int pt) {
     return (size_t)(MODE == WAVE_ITERATE ? 4 : 2) * CH * a.M * pt * sizeof(float);
   };
+  const bool cold = CH == 1 && a.L >= 200 && (MODE == WAVE_ITERATE || a.L < 260 || a.L >= 300);
+  const size_t least = cold ? 608 : 304;
   const auto fits = [&](int pt) {
-    return sm(pt) <= 72 * 1024 && (a.npix + pt - 1) / pt * a.B >= 304;
+    return sm(pt) <= 72 * 1024 && (a.npix + pt - 1) / pt * a.B >= least;
   };
   if (fits(64)) return launch_fold<CH, MODE, 64>(a, ctas_per_sm, sm(64), st, prof);
   if (fits(32)) return launch_fold<CH, MODE, 32>(a, ctas_per_sm, sm(32), st, prof);
-  return launch_fold<CH, MODE, 16>(a, ctas_per_sm, sm(16), st, prof);
+  return launch_narrow<CH, MODE>(a, ctas_per_sm, sm(16), st, prof);
 }
 
 FoldArgs base_args(const DctArgs &d) {
