@@ -544,6 +544,12 @@ __device__ __forceinline__ double image_scale(const ImageStat &t) {
   return t.nonfinite ? nan("") : (m > 0.f ? ldexp(1.0, -ilogbf(m)) : 1.0);
 }
 
+// the inverse of a scale, a power of two between 2^-127 and 2^149 (or NaN): from its
+// exponent, as a division a thread weighs on the FP64 pipe
+__device__ __forceinline__ double inverse_scale(double s) {
+  return s == s ? __hiloint2double((2046 - (__double2hiint(s) >> 20)) << 20, 0) : s;
+}
+
 struct Pairs {
   int n, L, per_cube;           // side, bands per cube, pairs per cube
   const ImageStat *stat;        // [images]
@@ -636,15 +642,20 @@ __global__ void k_pair_unpack(const double2 *__restrict__ z, double2 *__restrict
   const size_t N = (size_t)n * n, row = (size_t)kx * n;
   const double2 *zr = z + p * N + row, *zm = z + p * N + (size_t)((n - kx) & (n - 1)) * n;
   const bool two = P.second(p);
-  const double ra = 1.0 / P.scale(ia), rb = two ? 1.0 / P.scale(ia + 1) : 0.0;
+  const double ra = inverse_scale(P.scale(ia)), rb = two ? inverse_scale(P.scale(ia + 1)) : 0.0;
   const bool infa = P.infinite(ia), infb = two && P.infinite(ia + 1);
   const double2 inf = make_double2(HUGE_VAL, 0.0);
   double2 *ha = hh + ia * N + row, *hb = ha + N;
+  if (!two) {                                      // an odd last band: nothing to split
+    for (int ky = threadIdx.x; ky < n; ky += blockDim.x)
+      ha[ky] = infa ? inf : make_double2(ra * zr[ky].x, ra * zr[ky].y);
+    return;
+  }
   for (int ky = threadIdx.x; ky < n; ky += blockDim.x) {
     double2 A, B;
     pair_split(zr[ky], zm[(n - ky) & (n - 1)], A, B);
     ha[ky] = infa ? inf : make_double2(ra * A.x, ra * A.y);
-    if (two) hb[ky] = infb ? inf : make_double2(rb * B.x, rb * B.y);
+    hb[ky] = infb ? inf : make_double2(rb * B.x, rb * B.y);
   }
 }
 
