@@ -31,3 +31,19 @@ def test_fast_dct_batch_has_the_bits_of_a_cube_alone(n, L, B, sure):
                 p.solve(d, x[b], 6, [1e-2] * b if b > 1 else 1e-2, [2e-2] * b if b > 1 else 2e-2)
     for i in range(B):
         assert torch.equal(x[B][i], x[1][0]), i
+
+
+@pytest.mark.parametrize("n,L,J", [(32, 2, 3), (32, 8, 3), (16, 32, 2), (16, 64, 2), (8, 256, 2), (4, 1024, 2)])
+def test_default_precision_matches_oracle(n, L, J):
+    """The default spectral step of power-of-two band counts (the fast DCT,
+    tcgen05 for 64) in a plain solve; cube relative L2 1e-5."""
+    torch = cuda()
+    import paper_1905_08468_gb300 as pkg
+    from oracle import muffin as om
+    from tests.gpu_util import host, rel_l2
+    c = make_cube(n, L, max(2, n // 4), 1, 30 * n, seed=2100 + L)
+    x = torch.zeros((L, n, n), device="cuda")
+    with pkg.Plan(n, L, c.psf, n_wavelets=3, levels=J) as p:
+        p.solve(dev(c.dirty, torch), x, 20, 1e-2, 2e-2)
+    st, _ = om.solve(om.make_problem(c.dirty, c.psf, n_wavelets=3, J=J), 1e-2, 2e-2, 20)
+    assert rel_l2(host(x), st.x) <= 1e-5
