@@ -201,8 +201,9 @@ MUFFIN_API muffin_status muffin_plan_weights_from_x0(muffin_plan plan, const flo
  *   syn_packed       bit 0: coarse wavelet synthesis levels, bit 1: level 1;
  *                    0 = scalar row pass (one pixel row per thread),
  *                    1 = packed row pass (two rows per fma.rn.f32x2);
- *   dct_ctas_per_sm  CTAs per SM of the persistent spectral kernel
- *                    (0 = as many as fit).
+ *   dct_ctas_per_sm  CTAs per SM of a persistent grid of the dense spectral
+ *                    kernel (0 = a CTA per tile); without effect where
+ *                    another spectral kernel runs.
  * Which is fastest depends on the cube shape and the GPU. */
 typedef struct {
   int32_t syn_packed;      /* chosen synthesis variant bits */

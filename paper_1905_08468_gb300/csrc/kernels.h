@@ -91,7 +91,7 @@ int set_last_error_code(int s, const char *msg);
 // ------------------------------------------------------------ FFT (fft_conv.cu)
 // FP32 gradient pipeline: g[c][l] = H_l^T H_l x[c][l] - (c == 0 && b ? b[l] : 0)
 // for nimg = C*L images.  S: spectrum scratch [nimg][n/2+1][n] float2.
-// kspec: [L][n/2+1][n] = |h_hat_l(ky, kx)|^2 / n^2 (kx-major).
+// kspec: [L][n/2+1][n] = |h_hat_l(ky, kx)|^2 / n^2 (kx-major, ky in make_kspec's order).
 // chunk > 0: the three passes run over `chunk` images at a time (the
 // part of S that is used stays in L2 between the passes);
 // chunk <= 0: each pass over all images at once.

@@ -127,7 +127,10 @@ muffin_status validate(const muffin_params *p) {
                 "[2, 1024] (got %d)", p->nbands);
   if (!(p->tau >= 0) || !std::isfinite(p->tau))
     return fail(MUFFIN_EINVAL, "tau must be finite and >= 0 (0: from the step rule)");
-  // the spectral tile kernel keeps two [C][Lp][24] float tiles in shared memory
+  // the largest band count of a default-precision plan: the accepted range, kept as it
+  // was for every spectral kernel (two [C][Lp][24] float tiles in 200 KB); the dense
+  // kernel's narrowest tile, 4 C ceil(L / 2) 16 floats, fits throughout (132 KB at the
+  // range's ends, 1056 bands plain and 352 with ADA-PT)
   const size_t lp = (size_t)(p->nbands + 15) / 16 * 16;
   if (p->precision == 0 && (size_t)2 * (p->sure ? 3 : 1) * lp * 24 * sizeof(float) > 200 * 1024)
     return fail(MUFFIN_EINVAL, "nbands=%d too large for the spectral tile (sure=%d)",

@@ -92,7 +92,7 @@ struct muffin_plan_s {
   int syn_packed = 0;     // synthesis variant bits (see WaveArgs::syn_packed)
   int ana_ring = 0;       // kept for stored schedules, no effect
   int ana_pipe = 0;       // analysis tile height (see WaveArgs::ana_pipe)
-  int dct_ctas = 0;       // spectral kernel CTAs per SM (0: all resident)
+  int dct_ctas = 0;       // dense spectral kernel: CTAs per SM (0: a CTA per tile)
   int dct_tc = 0;         // spectral step on tcgen05 (L = 64)
   int grad_chunk = 0;     // images per pass of the gradient FFTs (0: all at once)
   int fft_radix = 16;     // largest radix of the gradient FFT plan (16, or 8 from n = 64)
